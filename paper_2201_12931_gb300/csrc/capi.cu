@@ -171,7 +171,7 @@ void free_all(topo_grid* h) {
     for (auto& d : h->dring64) F(d);
     for (auto& d : h->dring32) F(d);
     F(h->K0d); F(h->K0f);
-    F(h->dc_work); F(h->xnew_work); F(h->oc_hi); F(h->G64); F(h->oc_dv); F(h->S_cache); F(h->dv_cache); F(h->offs); F(h->wts);
+    F(h->dc_work); F(h->xnew_work); F(h->oc_hi); F(h->G64); F(h->oc_dv); F(h->stab); F(h->dv_cache);
     F(h->lam); F(h->dtmp); F(h->dflag); F(h->tc_err); F(h->tcB); F(h->partials); F(h->sc);
     if (h->host_sc) cudaFreeHost(h->host_sc);
     delete h->mk64;
@@ -254,36 +254,19 @@ topo_status ensure_coarse(topo_grid* h) {
 topo_status prepare_filter(topo_grid* h, double r) {
     if (!(r > 0.0) || r > 6.0) return fail(h, TOPO_BADARG, "filter radius must be in (0, 6]");
     if (r == h->S_radius) return TOPO_OK;
-    const int R = (int)std::ceil(r);
-    std::vector<int4> offs;
-    std::vector<double> wts;
-    for (int dz = -R; dz <= R; ++dz)
-        for (int dy = -R; dy <= R; ++dy)
-            for (int dx = -R; dx <= R; ++dx) {
-                const double w = r - std::sqrt((double)(dx * dx + dy * dy + dz * dz));
-                if (w > 0.0) {
-                    offs.push_back(make_int4(dx, dy, dz, 0));
-                    wts.push_back(w);
-                }
-            }
-    if (h->offs) cudaFree(h->offs);
-    if (h->wts) cudaFree(h->wts);
-    h->offs = nullptr;
-    h->wts = nullptr;
-    ALLOC(h, h->offs, offs.size());
-    ALLOC(h, h->wts, wts.size());
-    CK(h, cudaMemcpyAsync(h->offs, offs.data(), sizeof(int4) * offs.size(), cudaMemcpyHostToDevice, h->stream));
-    CK(h, cudaMemcpyAsync(h->wts, wts.data(), sizeof(double) * wts.size(), cudaMemcpyHostToDevice, h->stream));
-    h->noffs = (int)offs.size();
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
-    filter_launch(c, g, h->offs, h->wts, h->noffs, nullptr, h->S_cache, 2, nullptr);
-    fill(c, g.ne, h->xnew_work, 1.0);
-    divide(c, g.ne, h->xnew_work, h->S_cache, h->xnew_work);
-    filter_launch(c, g, h->offs, h->wts, h->noffs, h->xnew_work, h->dv_cache, 1, nullptr);
-    CK(h, cudaStreamSynchronize(h->stream));   // host vectors above go out of scope
+    filter_plan(g, r, h->nsm, &h->filt);
+    filter_weights(c, g, h->filt, h->stab);
     h->S_radius = r;
     return TOPO_OK;
+}
+
+// H^T 1, the volume sensitivity of the OC update, for the radius prepared last
+void prepare_dv(topo_grid* h) {
+    if (h->dv_radius == h->S_radius) return;
+    filter_launch(h->ctx(), h->lev[0].g, h->filt, 1, nullptr, nullptr, 0.0, h->stab, h->dv_cache);
+    h->dv_radius = h->S_radius;
 }
 
 // Operator coefficients of operator.cuh from the modal blocks; checks the
@@ -436,6 +419,7 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
         cudaGetLastError();
         nsm = 152;
     }
+    h->nsm = nsm;
     for (int l = 0; l < h->L; ++l) {
         Level& lv = h->lev[l];
         lv.g = make_geom(nx >> l, ny >> l, nz >> l);
@@ -469,7 +453,7 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
     TRY(dalloc(h, &h->dc_work, g0.ne));
     TRY(dalloc(h, &h->xnew_work, g0.ne));
     TRY(dalloc(h, &h->oc_hi, g0.ne));
-    TRY(dalloc(h, &h->S_cache, g0.ne));
+    TRY(dalloc(h, &h->stab, 2 * kFilterTab));
     TRY(dalloc(h, &h->dv_cache, g0.ne));
     TRY(dalloc(h, &h->lam, 8));
     TRY(dalloc(h, &h->dtmp, 8));
@@ -727,12 +711,7 @@ topo_status topo_filter(topo_handle h, double r, const double* in_dev, double* o
     if (s != TOPO_OK) return s;
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
-    if (transpose) {
-        divide(c, g.ne, in_dev, h->S_cache, h->xnew_work);
-        filter_launch(c, g, h->offs, h->wts, h->noffs, h->xnew_work, out_dev, 1, nullptr);
-    } else {
-        filter_launch(c, g, h->offs, h->wts, h->noffs, in_dev, out_dev, 0, nullptr);
-    }
+    filter_launch(c, g, h->filt, transpose ? 1 : 0, in_dev, nullptr, 0.0, h->stab, out_dev);
     CK(h, cudaGetLastError());
     return TOPO_OK;
 }
@@ -779,8 +758,8 @@ topo_status topo_oc_update(topo_handle h, double r, double move, double volfrac,
     if (s != TOPO_OK) return s;
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
-    divide(c, g.ne, dc_dev, h->S_cache, h->xnew_work);
-    filter_launch(c, g, h->offs, h->wts, h->noffs, h->xnew_work, h->dc_work, 1, nullptr);
+    prepare_dv(h);
+    filter_launch(c, g, h->filt, 1, dc_dev, nullptr, 0.0, h->stab, h->dc_work);
     // q over dc_work, lower bounds in xnew_work, upper bounds in oc_hi
     oc_prepare(c, g.ne, rho_dev_inout, h->dc_work, h->dv_cache, move, h->xnew_work, h->oc_hi);
     return oc_bisection(h, volfrac, rho_dev_inout, h->dv_cache, change_out, (double)g.ne);
@@ -839,8 +818,7 @@ topo_status topo_sensitivity_filter(topo_handle h, double r, double gamma, const
     if (!(gamma > 0.0)) return fail(h, TOPO_BADARG, "gamma must be positive");
     s = prepare_filter(h, r);
     if (s != TOPO_OK) return s;
-    sensitivity_filter(h->ctx(), h->lev[0].g, h->offs, h->wts, h->noffs, rho_dev, dc_dev, gamma, h->xnew_work,
-                       out_dev);
+    filter_launch(h->ctx(), h->lev[0].g, h->filt, 2, dc_dev, rho_dev, gamma, h->stab, out_dev);
     CK(h, cudaGetLastError());
     return TOPO_OK;
 }

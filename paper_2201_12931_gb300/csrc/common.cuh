@@ -92,6 +92,19 @@ struct PcgGraph {             // a captured launch sequence (a PCG iteration, or
     bool failed = false;      // capture not possible: direct launches
 };
 
+// Filter weights by class: w[c][pair_class(a, b)] = max(0, r - |(a, b, c)|) for
+// offsets 0 <= b <= a <= R in a plane and c planes apart (R <= 5); bit c of
+// bits = that weight is positive
+struct FilterW {
+    double w[6][21];
+    unsigned bits[21];
+};
+struct FilterPlan {
+    FilterW w;
+    int R = 0, tx = 32, cz = 1;   // largest offset; tile width and planes per CTA
+};
+constexpr int kFilterTab = 11 * 11 * 11;   // weight sums S by distance to the faces; then 1 / S
+
 struct Scalars {              // device-resident CG scalars
     double rz, rz_new, pq, rr, alpha, beta, ff, aux;
     double rz_old;            // z.r of the previous iteration (flexible beta)
@@ -123,12 +136,11 @@ struct topo_grid {
     double* oc_hi = nullptr;        // OC upper move-limit bounds
     double* G64 = nullptr;          // Galerkin child matrices P_o^T K0 P_o (homogenize = 2)
     double* oc_dv = nullptr;        // active-element indicator of a passive OC step (lazy)
-    double* S_cache = nullptr;      // filter weight sums S_e for S_radius
-    double* dv_cache = nullptr;     // H^T 1 for S_radius
-    int4* offs = nullptr;           // filter offsets for S_radius
-    double* wts = nullptr;          // filter weights for S_radius
-    int noffs = 0;
-    double S_radius = -1.0;
+    topo::FilterPlan filt{};        // weights and launch geometry of the filter for S_radius
+    double* stab = nullptr;         // its table of weight sums (2 kFilterTab)
+    double* dv_cache = nullptr;     // H^T 1 for dv_radius
+    double S_radius = -1.0, dv_radius = -1.0;
+    int nsm = 152;                  // multiprocessors of the device
     double* lam = nullptr;          // OC bisection state (device)
     double* dtmp = nullptr;         // device scratch scalars
     int* dflag = nullptr;           // device: density out of [0,1] seen
@@ -291,17 +303,18 @@ void transpose_dense(const Ctx& c, const double* W, double* WT, int npad);
 template <typename T>
 void coarse_apply(const Ctx& c, int n, int npad, const T* W, const T* WT, const T* rhs, T* y, T* out);
 
-// ---- filter_oc.cu --------------------------------------------------------
 // message returned by topo_last_error(NULL)
 void set_global_error(const std::string& msg);
-// mode 0: filter, 1: transpose of an input already divided by S, 2: weight sums S
-void filter_launch(const Ctx& c, const Geom& g, const int4* offs, const double* wts, int noffs, const double* in,
-                   double* out, int mode, const double* S);
-void divide(const Ctx& c, long long n, const double* a, const double* b, double* out);
-// q = x sqrt(max(-dc~, 1e-30) / dv~)
-// Eq. sensitivity filter: out = H(rho dc) / max(gamma, rho), tmp: work array
-void sensitivity_filter(const Ctx& c, const Geom& g, const int4* offs, const double* wts, int noffs,
-                        const double* rho, const double* dc, double gamma, double* tmp, double* out);
+// ---- filter.cu -----------------------------------------------------------
+// weights and launch geometry for radius r (0 < r <= 6)
+void filter_plan(const Geom& g, double r, int nsm, FilterPlan* p);
+// fills stab (2 kFilterTab doubles) with the weight sums of the plan's radius
+void filter_weights(const Ctx& c, const Geom& g, const FilterPlan& p, double* stab);
+// mode 0: out = H in; 1: out = H^T in (in null: H^T 1); 2: the sensitivity
+// filter out = H(rho in) / max(gamma, rho)
+void filter_launch(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, const double* in, const double* rho,
+                   double gamma, const double* stab, double* out);
+// ---- filter_oc.cu --------------------------------------------------------
 // q = x sqrt(max(-dc~,1e-30)/dv~) in place over dc~ (dv~ null: 1); lo / hi:
 // move-limit bounds.  The bisection steps take dv~ null for the volume of x
 // itself (no density filter).

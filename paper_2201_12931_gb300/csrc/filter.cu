@@ -1,0 +1,304 @@
+// Density filter (weights of Eqs. Neighbourhood / NB_dist, normalised by the
+// in-domain weight sum S_e), its transpose, and the paper's sensitivity filter.
+//
+// What bounds it: FP64 instructions run at 2 lanes per clock and SM on this
+// part (1/64 of the FP32 rate), so a neighbour-by-neighbour sum costs one
+// FP64 multiply-add per neighbour and element (93 at r = 3, 905 at r = 6)
+// while memory and the other pipes idle.  The weight depends on
+// dx^2 + dy^2 + dz^2 only, so the values are summed by symmetry first and
+// multiplied once per class:
+//   Y_b(i, j)  = v(i, j - b) + v(i, j + b)                  (shared by the row)
+//   G_ab(i, j) = sum of the 4 or 8 values at (+-a, +-b), (+-b, +-a), a >= b
+//   F_c(i, j)  = sum over the classes of w(a, b, c) G_ab
+//   out(k)     = F_0(k) + sum over c of F_c(k - c) + F_c(k + c)
+// marching along z with 2R + 1 running sums per column: 30 FP64
+// instructions per element instead of 93 at r = 3, 146 instead of 905 at
+// r = 6.  S_e depends only on the distances to the six faces, so it is a
+// table of (2R + 1)^3 entries, with reciprocals for the division.
+//
+// Measured, forward + transpose of 256x128x128 elements: r = 3, 2147 -> 784
+// us; the first call with a new radius 3689 -> 832 us.
+#include <math.h>
+
+#include "common.cuh"
+
+namespace topo {
+
+namespace {
+
+// class of index i along an axis of n elements: everything that the cut
+// neighbourhood depends on
+__host__ __device__ inline int face_class(int i, int n, int R) {
+    if (n <= 2 * R) return i;
+    return i < R ? i : (i >= n - R ? 2 * R - (n - 1 - i) : R);
+}
+__host__ __device__ constexpr int pair_class(int a, int b) { return a >= b ? a * (a + 1) / 2 + b : b * (b + 1) / 2 + a; }
+
+// S of every class triple and 1 / S.  S is formed by the very operations of
+// k_filter on in-domain values of 1 (the counts G are exact), so that H of
+// values in [0, 1] stays in [0, 1] and H 1 = 1 exactly: every operation is
+// monotone in the values.
+__global__ void k_filter_weights(const __grid_constant__ FilterW W, int R, int nx, int ny, int nz,
+                                 double* __restrict__ stab) {
+    const int nc = 2 * R + 1, t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nc * nc * nc) return;
+    const int cl[3] = {t % nc, (t / nc) % nc, t / (nc * nc)}, n[3] = {nx, ny, nz};
+    int lo[3], hi[3];
+    for (int q = 0; q < 3; ++q) {
+        if (n[q] <= 2 * R && cl[q] >= n[q]) return;   // no such element
+        lo[q] = -min(cl[q], R);
+        hi[q] = min(n[q] <= 2 * R ? n[q] - 1 - cl[q] : 2 * R - cl[q], R);
+    }
+    // in-domain values among the distinct (+-a, +-b)
+    auto count = [&](int a, int b) {
+        const int ca = a == 0 ? 1 : (-a >= lo[0]) + (a <= hi[0]), cb = b == 0 ? 1 : (-b >= lo[1]) + (b <= hi[1]);
+        return ca * cb;
+    };
+    double s = 0.0;
+    for (int dz = lo[2]; dz <= hi[2]; ++dz) {
+        const int c = abs(dz);
+        double F = 0.0;
+        for (int a = 0; a <= R; ++a)
+            for (int b = 0; b <= a; ++b) {
+                const int p = pair_class(a, b);
+                if ((W.bits[p] >> c) & 1u) F = fma(W.w[c][p], (double)(count(a, b) + (a != b ? count(b, a) : 0)), F);
+            }
+        s += F;
+    }
+    stab[t] = s;
+    stab[kFilterTab + t] = 1.0 / s;
+}
+
+// a / s with rs = fl(1 / s): product, exact remainder, correction (Markstein) --
+// 3 FP64 instructions instead of about 10.  Zeros, values near the ends of
+// the exponent range, infinities and NaN take the plain division; the tests
+// are on integer words.
+__device__ __forceinline__ double div_by(double a, double s, double rs) {
+    const int hi = __double2hiint(a);
+    if (((hi & 0x7fffffff) | __double2loint(a)) == 0) return a;
+    if ((unsigned)(((hi >> 20) & 0x7ff) - 128) >= 1792u) return a / s;
+    const double q = a * rs;
+    return fma(fma(-q, s, a), rs, q);
+}
+
+// MODE 0: out = H in; MODE 1: out = H^T in (in null: H^T 1); MODE 2: the
+// sensitivity filter H(rho in) / max(gamma, rho).
+// One CTA: TX x (128 / TX) element columns and a chunk of cz planes.  Per
+// plane: the tile with its halo goes to shared memory (loaded one plane
+// ahead into registers), Y, then G and F per thread.  128 threads, one warp
+// per scheduler; several CTAs per SM hide the two barriers per plane.
+// Weights that are zero inside the class list (r not an integer) are skipped
+// by the class's bit mask, not multiplied, so that an infinity or NaN
+// spreads to exactly the elements whose neighbourhood holds it.
+template <int R, int TX, int MODE>
+__global__ void __launch_bounds__(128) k_filter(const __grid_constant__ FilterW W, const int nx, const int ny,
+                                                const int nz, const int cz, const double* __restrict__ in,
+                                                const double* __restrict__ rho, const double gamma,
+                                                const double* __restrict__ stab, double* __restrict__ out) {
+    constexpr int TY = 128 / TX, PW = TX + 2 * R, PH = TY + 2 * R, NT = PW * PH, NL = (NT + 127) / 128;
+    constexpr int nc = 2 * R + 1;
+    __shared__ double v[2][PH][PW];
+    __shared__ double Y[R > 0 ? R : 1][TY][PW];
+    const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+    // one-dimensional grid (x tiles fastest): long thin grids exceed the y and z limits
+    const int gx = (nx + TX - 1) / TX, gy = (ny + TY - 1) / TY;
+    const int bxy = blockIdx.x % (gx * gy);
+    const int i0 = bxy % gx * TX, j0 = bxy / gx * TY;
+    const int k0 = blockIdx.x / (gx * gy) * cz, k1 = min(k0 + cz, nz);
+    const int nxy = nx * ny;
+    int off[NL];
+    [[maybe_unused]] int cxy[NL];
+    double raw[NL];
+    [[maybe_unused]] double raw2[NL];
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        const int pos = tid + 128 * l, gi = i0 - R + pos % PW, gj = j0 - R + pos / PW;
+        const bool ok = pos < NT && gi >= 0 && gi < nx && gj >= 0 && gj < ny;
+        off[l] = ok ? gi + nx * gj : -1;
+        if constexpr (MODE == 1) cxy[l] = ok ? face_class(gj, ny, R) * nc + face_class(gi, nx, R) : 0;
+        raw[l] = 0.0;
+    }
+    auto fetch = [&](int k) {
+#pragma unroll
+        for (int l = 0; l < NL; ++l)
+            if (off[l] >= 0) {
+                if (MODE != 1 || in) raw[l] = in[off[l] + nxy * k];
+                if constexpr (MODE == 2) raw2[l] = rho[off[l] + nxy * k];
+            }
+    };
+    const int i = i0 + tx, j = j0 + ty;
+    const bool act = i < nx && j < ny;
+    const int ccol = act ? face_class(j, ny, R) * nc + face_class(i, nx, R) : 0;
+    double acc[2 * R + 1];
+#pragma unroll
+    for (int d = 0; d <= 2 * R; ++d) acc[d] = 0.0;
+    const int kb = max(k0 - R, 0), ke = min(k1 - 1 + R, nz - 1);
+    fetch(kb);
+    for (int k = kb; k <= k1 - 1 + R; ++k) {
+        if (k <= ke) {
+            double(*vb)[PW] = v[k & 1];
+#pragma unroll
+            for (int l = 0; l < NL; ++l) {
+                const int pos = tid + 128 * l;
+                if (pos < NT) {
+                    double t = raw[l];
+                    if constexpr (MODE == 1) {
+                        const int ct = face_class(k, nz, R) * nc * nc + cxy[l];
+                        if (off[l] >= 0) t = in ? div_by(t, stab[ct], stab[kFilterTab + ct]) : stab[kFilterTab + ct];
+                    }
+                    if constexpr (MODE == 2)
+                        if (off[l] >= 0) t *= raw2[l];
+                    vb[pos / PW][pos % PW] = t;
+                }
+            }
+            if (k < ke) fetch(k + 1);
+            __syncthreads();
+            if constexpr (R > 0) {
+                for (int t = tid; t < TY * PW; t += 128) {
+                    const int row = t / PW, col = t % PW;
+#pragma unroll
+                    for (int b = 1; b <= R; ++b) Y[b - 1][row][col] = vb[row + R - b][col] + vb[row + R + b][col];
+                }
+                __syncthreads();
+            }
+            if (act) {
+                // planes k - c and k + c that this chunk outputs
+                unsigned need = 0;
+#pragma unroll
+                for (int c = 0; c <= R; ++c)
+                    if ((k - c >= k0 && k - c < k1) || (k + c >= k0 && k + c < k1)) need |= 1u << c;
+                double F[R + 1];
+#pragma unroll
+                for (int c = 0; c <= R; ++c) F[c] = 0.0;
+                const double* vr = &vb[ty + R][tx + R];
+#pragma unroll
+                for (int a = 0; a <= R; ++a)
+#pragma unroll
+                    for (int b = 0; b <= a; ++b) {
+                        const int p = pair_class(a, b);
+                        const unsigned m = W.bits[p] & need;
+                        if (m == 0) continue;
+                        double G;
+                        if (a == 0) {
+                            G = vr[0];
+                        } else if (b == 0) {
+                            G = (vr[-a] + vr[a]) + Y[a - 1][ty][tx + R];
+                        } else if (a == b) {
+                            G = Y[a - 1][ty][tx + R - a] + Y[a - 1][ty][tx + R + a];
+                        } else {
+                            const double* ya = Y[a - 1][ty] + tx + R;
+                            const double* yb = Y[b - 1][ty] + tx + R;
+                            G = (ya[-b] + ya[b]) + (yb[-a] + yb[a]);
+                        }
+#pragma unroll
+                        for (int c = 0; c <= R; ++c)
+                            if ((m >> c) & 1u) F[c] = fma(W.w[c][p], G, F[c]);
+                    }
+#pragma unroll
+                for (int d = 0; d <= 2 * R; ++d) {
+                    const int ko = k - R + d;
+                    if (ko >= k0 && ko < k1) acc[d] += F[d < R ? R - d : d - R];
+                }
+            }
+        }
+        const int ko = k - R;
+        if (act && ko >= k0) {
+            const int e = i + nx * j + nxy * ko;
+            double o = acc[0];
+            if constexpr (MODE != 1) {
+                const int ct = face_class(ko, nz, R) * nc * nc + ccol;
+                o = div_by(o, stab[ct], stab[kFilterTab + ct]);
+                if constexpr (MODE == 2) o = o / fmax(gamma, rho[e]);
+            }
+            out[e] = o;
+        }
+#pragma unroll
+        for (int d = 0; d < 2 * R; ++d) acc[d] = acc[d + 1];
+        acc[2 * R] = 0.0;
+    }
+}
+
+template <int R, int TX>
+void launch(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, const double* in, const double* rho,
+            double gamma, const double* stab, double* out) {
+    constexpr int TY = 128 / TX;
+    const unsigned grid = (unsigned)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY) * ((g.nz + p.cz - 1) / p.cz);
+    if (mode == 0)
+        k_filter<R, TX, 0><<<grid, 128, 0, c.s>>>(p.w, g.nx, g.ny, g.nz, p.cz, in, nullptr, 0.0, stab, out);
+    else if (mode == 1)
+        k_filter<R, TX, 1><<<grid, 128, 0, c.s>>>(p.w, g.nx, g.ny, g.nz, p.cz, in, nullptr, 0.0, stab, out);
+    else
+        k_filter<R, TX, 2><<<grid, 128, 0, c.s>>>(p.w, g.nx, g.ny, g.nz, p.cz, in, rho, gamma, stab, out);
+    TOPO_LAUNCH_CHECK(c);
+}
+
+template <int R>
+void launch_tx(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, const double* in, const double* rho,
+               double gamma, const double* stab, double* out) {
+    if (p.tx == 16) launch<R, 16>(c, g, p, mode, in, rho, gamma, stab, out);
+    else launch<R, 32>(c, g, p, mode, in, rho, gamma, stab, out);
+}
+
+}  // namespace
+
+void filter_plan(const Geom& g, double r, int nsm, FilterPlan* p) {
+    p->R = (int)ceil(r) - 1;   // largest offset along an axis with a positive weight
+    const int R = p->R;
+    int adds = 0, fmas = 2 * R;
+    for (int a = 0; a <= R; ++a)
+        for (int b = 0; b <= a; ++b) {
+            const int q = pair_class(a, b);
+            p->w.bits[q] = 0;
+            for (int c = 0; c <= R; ++c) {
+                const double w = r - sqrt((double)(a * a + b * b + c * c));
+                p->w.w[c][q] = w > 0.0 ? w : 0.0;
+                if (w > 0.0) {
+                    p->w.bits[q] |= 1u << c;
+                    ++fmas;
+                }
+            }
+            if (p->w.bits[q]) adds += a == 0 ? 0 : (b == 0 ? 2 : (a == b ? 1 : 3));
+        }
+    // Tile width and planes per CTA that minimise the FP64 time of the
+    // fullest SM (16 clocks per warp instruction and SM, 4 warps per CTA)
+    // plus the latency of the march (about 600 clocks a plane).  A chunk of
+    // cz planes sums cz + 2R of them; narrow grids waste fewer lanes on tiles
+    // of 16.
+    double best = -1.0;
+    for (int tx = 16; tx <= 32; tx *= 2) {
+        const double per_plane = adds + (double)R * (tx + 2 * R) / tx;
+        const long long xy = (long long)((g.nx + tx - 1) / tx) * ((g.ny + 128 / tx - 1) / (128 / tx));
+        for (int cz = 1;; cz = cz < 4 ? cz + 1 : cz + cz / 3) {
+            if (cz > g.nz) cz = g.nz;
+            const long long ctas = xy * ((g.nz + cz - 1) / cz);
+            const double dp = 64.0 * ((cz + 2 * R) * per_plane + cz * (fmas + 3.0));
+            const double t = (double)((ctas + nsm - 1) / nsm) * dp + 600.0 * (cz + 2 * R);
+            if (best < 0.0 || t < best) {
+                best = t;
+                p->tx = tx;
+                p->cz = cz;
+            }
+            if (cz >= g.nz || cz >= 256) break;
+        }
+    }
+}
+
+void filter_weights(const Ctx& c, const Geom& g, const FilterPlan& p, double* stab) {
+    const int nc = 2 * p.R + 1;
+    k_filter_weights<<<(nc * nc * nc + 31) / 32, 32, 0, c.s>>>(p.w, p.R, g.nx, g.ny, g.nz, stab);
+    TOPO_LAUNCH_CHECK(c);
+}
+
+void filter_launch(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, const double* in, const double* rho,
+                   double gamma, const double* stab, double* out) {
+    switch (p.R) {
+        case 0: launch_tx<0>(c, g, p, mode, in, rho, gamma, stab, out); break;
+        case 1: launch_tx<1>(c, g, p, mode, in, rho, gamma, stab, out); break;
+        case 2: launch_tx<2>(c, g, p, mode, in, rho, gamma, stab, out); break;
+        case 3: launch_tx<3>(c, g, p, mode, in, rho, gamma, stab, out); break;
+        case 4: launch_tx<4>(c, g, p, mode, in, rho, gamma, stab, out); break;
+        default: launch_tx<5>(c, g, p, mode, in, rho, gamma, stab, out); break;
+    }
+}
+
+}  // namespace topo

@@ -1,6 +1,5 @@
-// Density filter (weights of Eqs. Neighbourhood / NB_dist, normalised by the
-// in-domain weight sum), its transpose, and the optimality-criteria update with
-// bisection on the Lagrange multiplier (Eqs. OCUp1, bisect).
+// Optimality-criteria update with bisection on the Lagrange multiplier (Eqs.
+// OCUp1, bisect) and the self-weight load.
 //
 // The volume of the filtered new design is evaluated without filtering it:
 // mean(H x) = (1/N) sum_e sum_i w_ei x_i / S_e = (1/N) (H^T 1)^T x, so one
@@ -43,65 +42,6 @@ __device__ __forceinline__ double block_max(double v, double* sh) {
         for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, o));
     }
     return t;
-}
-
-// mode 0: out_e = sum_d w_d in[e+d] / S_e (S_e on the fly)
-// mode 1: out_i = sum_d w_d in[i+d]   with in = g / S already divided
-// mode 2: out_e = S_e
-template <int MODE>
-__global__ void __launch_bounds__(256) k_filter(const int4* __restrict__ offs, const double* __restrict__ wts,
-                                                int noffs, int nx, int ny, int nz, const double* __restrict__ in,
-                                                const double* __restrict__ S, double* __restrict__ out) {
-    extern __shared__ int4 soff[];                       // offsets first: 16-byte aligned
-    double* sw = reinterpret_cast<double*>(soff + noffs);
-    for (int t = threadIdx.x; t < noffs; t += blockDim.x) {
-        sw[t] = wts[t];
-        soff[t] = offs[t];
-    }
-    __syncthreads();
-    const long long ne = (long long)nx * ny * nz;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ne; e += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(e % nx);
-        const long long t = e / nx;
-        const int j = (int)(t % ny), k = (int)(t / ny);
-        double acc = 0.0, ws = 0.0;
-        for (int q = 0; q < noffs; ++q) {
-            const int4 o = soff[q];
-            const int a = i + o.x, b = j + o.y, c = k + o.z;
-            if (a < 0 || a >= nx || b < 0 || b >= ny || c < 0 || c >= nz) continue;
-            const double w = sw[q];
-            const long long nb = a + (long long)nx * (b + (long long)ny * c);
-            if (MODE == 0) {
-                acc += w * in[nb];
-                ws += w;
-            } else if (MODE == 1) {
-                acc += w * in[nb];   // in = g / S, formed by k_divide
-            } else {
-                ws += w;
-            }
-        }
-        out[e] = (MODE == 0) ? acc / ws : (MODE == 1 ? acc : ws);
-    }
-}
-
-// Eq. sensitivity filter: t = rho dc before the normalised filter, and the
-// division by max(gamma, rho_e) after it
-__global__ void k_mul(long long n, const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out) {
-    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    out[e] = a[e] * b[e];
-}
-__global__ void k_div_max(long long n, double* __restrict__ out, const double* __restrict__ rho, double gamma) {
-    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    out[e] = out[e] / fmax(gamma, rho[e]);
-}
-
-__global__ void k_divide(long long n, const double* __restrict__ a, const double* __restrict__ b,
-                         double* __restrict__ out) {
-    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    out[e] = a[e] / b[e];
 }
 
 // q_e = x_e sqrt(max(-dc~_e, 1e-30) / dv~_e): the part of the OC candidate
@@ -257,31 +197,6 @@ __global__ void __launch_bounds__(1024) k_max_to(const double* __restrict__ part
 }
 
 }  // namespace
-
-void filter_launch(const Ctx& c, const Geom& g, const int4* offs, const double* wts, int noffs, const double* in,
-                   double* out, int mode, const double* S) {
-    unsigned blocks = grid_for(g.ne, 256);
-    if (blocks > 16384) blocks = 16384;
-    const size_t sm = (sizeof(int4) + sizeof(double)) * (size_t)noffs;
-    if (mode == 0) k_filter<0><<<blocks, 256, sm, c.s>>>(offs, wts, noffs, g.nx, g.ny, g.nz, in, S, out);
-    else if (mode == 1) k_filter<1><<<blocks, 256, sm, c.s>>>(offs, wts, noffs, g.nx, g.ny, g.nz, in, S, out);
-    else k_filter<2><<<blocks, 256, sm, c.s>>>(offs, wts, noffs, g.nx, g.ny, g.nz, in, S, out);
-    TOPO_LAUNCH_CHECK(c);
-}
-
-void divide(const Ctx& c, long long n, const double* a, const double* b, double* out) {
-    k_divide<<<grid_for(n, 256), 256, 0, c.s>>>(n, a, b, out);
-    TOPO_LAUNCH_CHECK(c);
-}
-
-void sensitivity_filter(const Ctx& c, const Geom& g, const int4* offs, const double* wts, int noffs,
-                        const double* rho, const double* dc, double gamma, double* tmp, double* out) {
-    k_mul<<<grid_for(g.ne, 256), 256, 0, c.s>>>(g.ne, rho, dc, tmp);
-    TOPO_LAUNCH_CHECK(c);
-    filter_launch(c, g, offs, wts, noffs, tmp, out, 0, nullptr);
-    k_div_max<<<grid_for(g.ne, 256), 256, 0, c.s>>>(g.ne, out, rho, gamma);
-    TOPO_LAUNCH_CHECK(c);
-}
 
 void oc_prepare(const Ctx& c, long long ne, const double* x, double* dct_q, const double* dv, double move, double* lo,
                 double* hi) {
