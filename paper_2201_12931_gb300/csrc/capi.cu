@@ -172,7 +172,7 @@ void free_all(topo_grid* h) {
     for (auto& d : h->dring32) F(d);
     F(h->K0d); F(h->K0f);
     F(h->dc_work); F(h->xnew_work); F(h->oc_hi); F(h->G64); F(h->oc_dv); F(h->stab); F(h->dv_cache);
-    F(h->lam); F(h->dtmp); F(h->dflag); F(h->tc_err); F(h->tcB); F(h->partials); F(h->sc);
+    F(h->lam); F(h->oc_ws); F(h->dtmp); F(h->dflag); F(h->tc_err); F(h->tcB); F(h->partials); F(h->sc);
     if (h->host_sc) cudaFreeHost(h->host_sc);
     delete h->mk64;
     delete h->mk32;
@@ -718,32 +718,49 @@ topo_status topo_filter(topo_handle h, double r, const double* in_dev, double* o
 
 // bisection of Eq. OC on lambda (reading of the paper: l1 = 0, l2 = 1e9,
 // relative tolerance 1e-9) over q = x sqrt(-dc / dv) in dc_work and the
-// bounds in xnew_work / oc_hi; dv null: volume of x itself; writes x and change
+// bounds in xnew_work / oc_hi; dv null: volume of x itself; writes x and change.
+// The search (oc_search) finds the same multiplier from a few passes; values
+// that it does not cover (negative or NaN entries, no root in its range, too
+// many elements at a bound in its last bracket) take one pass over all
+// elements per bisection step.
 static topo_status oc_bisection(topo_grid* h, double volfrac, double* rho_dev_inout, const double* dv,
                                 double* change_out, double n_volume) {
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
     const double l1 = 0.0, l2 = 1e9, tol = 1e-9;
-    const double init[8] = {l1, l2, 0.5 * (l1 + l2), (l2 - l1) / (l1 + l2) > tol ? 0.0 : 1.0, 0.0, 0.5 * (l1 + l2),
-                            0.0, 0.0};
-    CK(h, cudaMemcpyAsync(h->lam, init, sizeof(init), cudaMemcpyHostToDevice, h->stream));
-    double state[8];
-    for (int batch = 0; batch < 25; ++batch) {
-        for (int k = 0; k < 16; ++k) {
-            oc_bisect_step(c, g.ne, h->xnew_work, h->oc_hi, h->dc_work, dv, h->partials, h->lam);
-            oc_bisect_finalize(c, h->partials, h->lam, volfrac * n_volume, tol);
+    double change = 0.0;
+    bool bad = false;
+    oc_search(c, g.ne, h->xnew_work, h->oc_hi, h->dc_work, dv, h->r, h->oc_ws, volfrac * n_volume, tol);
+    oc_search_write(c, g.ne, rho_dev_inout, h->xnew_work, h->oc_hi, h->dc_work, h->oc_ws, h->partials);
+    CK(h, oc_search_read(c, h->oc_ws, &change, &bad));
+    if (bad) {
+        const double init[8] = {l1, l2, 0.5 * (l1 + l2), (l2 - l1) / (l1 + l2) > tol ? 0.0 : 1.0, 0.0,
+                                0.5 * (l1 + l2), 0.0, 0.0};
+        CK(h, cudaMemcpyAsync(h->lam, init, sizeof(init), cudaMemcpyHostToDevice, h->stream));
+        double state[8];
+        for (int batch = 0; batch < 25; ++batch) {
+            for (int k = 0; k < 16; ++k) {
+                oc_bisect_step(c, g.ne, h->xnew_work, h->oc_hi, h->dc_work, dv, h->partials, h->lam);
+                oc_bisect_finalize(c, h->partials, h->lam, volfrac * n_volume, tol);
+            }
+            CK(h, cudaMemcpyAsync(state, h->lam, sizeof(state), cudaMemcpyDeviceToHost, h->stream));
+            CK(h, cudaStreamSynchronize(h->stream));
+            if (state[3] != 0.0) break;
         }
-        CK(h, cudaMemcpyAsync(state, h->lam, sizeof(state), cudaMemcpyDeviceToHost, h->stream));
-        CK(h, cudaStreamSynchronize(h->stream));
-        if (state[3] != 0.0) break;
+        if (state[3] == 0.0) return fail(h, TOPO_MAXITER, "bisection did not converge");
+        oc_write(c, g.ne, rho_dev_inout, h->xnew_work, h->oc_hi, h->dc_work, h->lam, h->oc_ws, h->partials);
+        CK(h, oc_search_read(c, h->oc_ws, &change, &bad));
     }
-    if (state[3] == 0.0) return fail(h, TOPO_MAXITER, "bisection did not converge");
-    oc_write(c, g.ne, rho_dev_inout, h->xnew_work, h->oc_hi, h->dc_work, h->lam, h->partials, h->dtmp);
-    if (change_out) {
-        CK(h, cudaMemcpyAsync(change_out, h->dtmp, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-        CK(h, cudaStreamSynchronize(h->stream));
-    }
+    if (change_out) *change_out = change;
     CK(h, cudaGetLastError());
+    return TOPO_OK;
+}
+
+// workspace of the search: its state, and packed FP32 copies of the element
+// data in the FP64 residual vector, which holds nothing between calls (24 B
+// per node against 16 B per element)
+static topo_status ensure_oc(topo_grid* h) {
+    if (!h->oc_ws) ALLOC(h, h->oc_ws, oc_search_bytes());
     return TOPO_OK;
 }
 
@@ -756,12 +773,15 @@ topo_status topo_oc_update(topo_handle h, double r, double move, double volfrac,
         return fail(h, TOPO_BADARG, "move must be in (0,1], volfrac in (0,1)");
     s = prepare_filter(h, r);
     if (s != TOPO_OK) return s;
+    s = ensure_oc(h);
+    if (s != TOPO_OK) return s;
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
     prepare_dv(h);
     filter_launch(c, g, h->filt, 1, dc_dev, nullptr, 0.0, h->stab, h->dc_work);
     // q over dc_work, lower bounds in xnew_work, upper bounds in oc_hi
-    oc_prepare(c, g.ne, rho_dev_inout, h->dc_work, h->dv_cache, move, h->xnew_work, h->oc_hi);
+    oc_prepare(c, g.ne, rho_dev_inout, h->dc_work, h->dc_work, h->dv_cache, nullptr, move, h->xnew_work, h->oc_hi,
+               h->r, h->oc_ws);
     return oc_bisection(h, volfrac, rho_dev_inout, h->dv_cache, change_out, (double)g.ne);
 }
 
@@ -772,15 +792,14 @@ topo_status topo_oc_update_unfiltered(topo_handle h, double move, double volfrac
     if (!rho_dev_inout || !dc_dev) return fail(h, TOPO_BADARG, "NULL pointer");
     if (!(move > 0.0 && move <= 1.0) || !(volfrac > 0.0 && volfrac < 1.0))
         return fail(h, TOPO_BADARG, "move must be in (0,1], volfrac in (0,1)");
+    s = ensure_oc(h);
+    if (s != TOPO_OK) return s;
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
-    CK(h, cudaMemcpyAsync(h->dc_work, dc_dev, sizeof(double) * g.ne, cudaMemcpyDeviceToDevice, h->stream));
-    if (!passive_dev) {
-        oc_prepare(c, g.ne, rho_dev_inout, h->dc_work, nullptr, move, h->xnew_work, h->oc_hi);
-        return oc_bisection(h, volfrac, rho_dev_inout, nullptr, change_out, (double)g.ne);
-    }
-    if (!h->oc_dv) ALLOC(h, h->oc_dv, g.ne);
-    oc_prepare_passive(c, g.ne, rho_dev_inout, h->dc_work, passive_dev, move, h->xnew_work, h->oc_hi, h->oc_dv);
+    if (passive_dev && !h->oc_dv) ALLOC(h, h->oc_dv, g.ne);
+    oc_prepare(c, g.ne, rho_dev_inout, dc_dev, h->dc_work, passive_dev ? h->oc_dv : nullptr, passive_dev, move,
+               h->xnew_work, h->oc_hi, h->r, h->oc_ws);
+    if (!passive_dev) return oc_bisection(h, volfrac, rho_dev_inout, nullptr, change_out, (double)g.ne);
     dot_partials<double, double>(c, g.ne, h->oc_dv, h->oc_dv, h->partials);   // number of active elements
     reduce_to(c, h->partials, kRedBlocks, h->dtmp);
     double n_active = 0.0;

@@ -142,6 +142,7 @@ struct topo_grid {
     double S_radius = -1.0, dv_radius = -1.0;
     int nsm = 152;                  // multiprocessors of the device
     double* lam = nullptr;          // OC bisection state (device)
+    char* oc_ws = nullptr;          // search for the OC multiplier (oc_search_bytes, on first use)
     double* dtmp = nullptr;         // device scratch scalars
     int* dflag = nullptr;           // device: density out of [0,1] seen
     bool coarse_dirty = true;
@@ -314,16 +315,24 @@ void filter_weights(const Ctx& c, const Geom& g, const FilterPlan& p, double* st
 // filter out = H(rho in) / max(gamma, rho)
 void filter_launch(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, const double* in, const double* rho,
                    double gamma, const double* stab, double* out);
-// ---- filter_oc.cu --------------------------------------------------------
-// q = x sqrt(max(-dc~,1e-30)/dv~) in place over dc~ (dv~ null: 1); lo / hi:
-// move-limit bounds.  The bisection steps take dv~ null for the volume of x
-// itself (no density filter).
-void oc_prepare(const Ctx& c, long long ne, const double* x, double* dct_q, const double* dv, double move, double* lo,
-                double* hi);
-// passive elements (0 active, 1 solid, 2 void): lo = hi = 1 / 0, q = 0,
-// dv = 0; active: q = x sqrt(max(-dc, 1e-30)), move-limit bounds, dv = 1
-void oc_prepare_passive(const Ctx& c, long long ne, const double* x, double* dct_q, const uint8_t* passive,
-                        double move, double* lo, double* hi, double* dv);
+// ---- oc.cu ---------------------------------------------------------------
+// OC update: q = x sqrt(max(-dc~, 1e-30) / dv~) (in place over dc~ allowed),
+// move-limit bounds lo / hi, and FP32 copies of (q, lo, hi, dv) in pack (16 B
+// per element).  dv null: 1 (the volume of x itself); passive (0 active, 1
+// solid, 2 void): lo = hi = 1 / 0, q = 0, and dv is written (0; active: 1).
+void oc_prepare(const Ctx& c, long long ne, const double* x, const double* dct, double* q, double* dv,
+                const uint8_t* passive, double move, double* lo, double* hi, void* pack, void* search);
+// the multiplier with sum dv clamp(q lambda^(-1/2), lo, hi) = target: screening
+// passes in FP32, then the bisection on [0, 1e9] with exact volumes; result
+// and success in the search state (oc_search_bytes of device memory)
+size_t oc_search_bytes();
+void oc_search(const Ctx& c, long long ne, const double* lo, const double* hi, const double* q, const double* dv,
+               const void* pack, void* search, double target, double tol);
+// x_new of a successful search (x untouched else), then the change and
+// whether the search failed (synchronises)
+void oc_search_write(const Ctx& c, long long ne, double* x, const double* lo, const double* hi, const double* q,
+                     void* search, double* partials);
+cudaError_t oc_search_read(const Ctx& c, const void* search, double* change, bool* bad);
 // self-weight load f_out = f_ext (null: 0) - (w/8) sum of rho over the elements at each node, in z
 void gravity_load(const Ctx& c, const Geom& g, const double* rho, const double* f_ext, double* f_out, double w);
 // dc_e += -(w/4) sum of u_z over the corners of e
@@ -332,8 +341,8 @@ void oc_bisect_step(const Ctx& c, long long ne, const double* lo, const double* 
                     const double* dv, double* partials, double* lam_state);
 void oc_bisect_finalize(const Ctx& c, const double* partials, double* lam_state, double volfrac_ne,
                         double tol);
-void oc_write(const Ctx& c, long long ne, double* x, const double* lo, const double* hi, const double* num,
-              const double* lam_state, double* partials, double* change_dst);
+void oc_write(const Ctx& c, long long ne, double* x, const double* lo, const double* hi, const double* q,
+              const double* lam_state, void* search, double* partials);
 
 }  // namespace topo
 

@@ -1,0 +1,36 @@
+// FP64 helpers in few FP64 instructions.  FP64 instructions and FP64 <-> FP32
+// conversions run at 2 lanes per clock and SM on this part, 1/64 of the
+// integer and FP32 rates, so conversions go through integer words and the
+// iterations start from an FP32 seed.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace topo {
+
+// FP32 value of a non-negative double, truncated (relative error below 2^-23;
+// 0 below FP32's normal range, infinity above)
+__device__ __forceinline__ float trunc_f32(double v) {
+    const int hi = __double2hiint(v);
+    if (hi < (897 << 20)) return 0.0f;
+    if (hi >= (1151 << 20)) return __int_as_float(0x7f800000);
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(v), (unsigned)hi, 3) - 0xc0000000u);
+}
+// a positive normal FP32 value, exactly
+__device__ __forceinline__ double widen_f32(float v) {
+    const unsigned b = __float_as_uint(v);
+    return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+}
+// 1 / b by two Newton steps from the FP32 reciprocal, for 2^-100 <= b < 2^100
+__device__ __forceinline__ double recip_seeded(double b) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(trunc_f32(b)));
+    double y = widen_f32(r);
+    y = fma(fma(-b, y, 1.0), y, y);
+    return fma(fma(-b, y, 1.0), y, y);
+}
+__device__ __forceinline__ bool seed_range(double b) {
+    return (unsigned)((__double2hiint(b) >> 20) - (1023 - 100)) < 200u;
+}
+
+}  // namespace topo
