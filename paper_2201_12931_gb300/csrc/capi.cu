@@ -128,6 +128,9 @@ topo_status alloc_precision(topo_grid* h, bool fp64) {
         ALLOC(h, h->p, n0);
         ALLOC(h, h->q, n0);
         for (auto& d : h->dring64) ALLOC(h, d, n0);
+        size_t el = 0;
+        for (auto& lv : h->lev) el = std::max(el, lv.p64.scratch());
+        if (el > 0) ALLOC(h, h->el64, el);
         h->fp64_ready = true;
     } else {
         ALLOC(h, h->r32, n0);
@@ -167,7 +170,7 @@ void free_all(topo_grid* h) {
     F(h->cs.A); F(h->cs.W64); F(h->cs.WT64); F(h->cs.W32); F(h->cs.WT32); F(h->cs.y64); F(h->cs.y32);
     F(h->cs.info); F(h->cs.Dk);
     F(h->x); F(h->f); F(h->r); F(h->z); F(h->p); F(h->q);
-    F(h->r32); F(h->z32); F(h->p32); F(h->q32); F(h->d32); F(h->alpha_hist);
+    F(h->r32); F(h->z32); F(h->p32); F(h->q32); F(h->d32); F(h->alpha_hist); F(h->el64);
     for (auto& d : h->dring64) F(d);
     for (auto& d : h->dring32) F(d);
     F(h->K0d); F(h->K0f);
@@ -427,6 +430,8 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
         lv.op32 = op_launch32(lv.g, nsm);
         lv.op64 = op_launch64(lv.g, nsm);
         lv.optc = op_launch_tc(lv.g, nsm);
+        if (lv.g.ne <= kOp64Max) lv.p64 = op64_plan(lv.g, nsm);
+        h->npartials = std::max(h->npartials, (long long)lv.p64.blocks);
         h->npartials = std::max(h->npartials, std::max(lv.op32.ctas(), std::max(lv.op64.ctas(), lv.optc.ctas())));
     }
     topo_status st;
@@ -906,6 +911,7 @@ static topo_status level_op(topo_grid* h, int level, int precision, int op, cons
         if (stencil_df(c, mode, lv.op64, *h->mkdf, lv.E64, lv.mask, u, f, out, nullptr, nullptr) < 0)
             return fail(h, TOPO_BADARG, "double-FP32 kernel: mode not available");
     } else if (precision == TOPO_FP64) {
+        if (op == OP_JACOBI) ensure_dinv64(h);
         op_apply<double>(h, mode, level, u, f, out, nullptr);
     } else {
         convert<double, float>(c, n, u, lv.v32.a);

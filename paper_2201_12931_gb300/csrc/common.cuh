@@ -42,6 +42,13 @@ struct OpLaunch {          // launch geometry of the operator kernel on one leve
     long long ctas() const { return (long long)gx * gy * gz; }
 };
 
+struct Op64Plan {          // FP64 operator by elements (op64.cu)
+    int cz = 0;            // layers per thread; 0: the level uses the tile kernel
+    int blocks = 0;        // blocks of the node kernel (dot partials)
+    long long nt = 0;      // element threads
+    size_t scratch() const { return (size_t)(cz + 1) * 12 * nt; }   // doubles
+};
+
 template <typename T>
 struct ModalK;
 
@@ -60,6 +67,7 @@ struct Level {
     float* Ke32 = nullptr;
     OpLaunch op32, op64;      // operator launch geometry per precision
     OpLaunch optc;            // tensor-core FP32 operator (tc_op.cu)
+    Op64Plan p64;             // FP64 operator by elements (op64.cu)
     double scale = 1.0;       // 2^l
     double* rho = nullptr;    // homogenized density
     double* E64 = nullptr;    // 2^l * (Emin + rho^p (E0 - Emin))
@@ -164,6 +172,7 @@ struct topo_grid {
     double* dring64[topo::kDirRing - 2] = {};
     float* dring32[topo::kDirRing - 2] = {};
     double* alpha_hist = nullptr;   // device: alpha of each ring slot
+    double* el64 = nullptr;         // face contributions of the FP64 operator by elements (op64.cu)
     topo::PcgGraph graph64[topo::kDirRing], graph32[topo::kDirRing];   // captured PCG iterations per ring slot
     topo::PcgGraph coarse_graph;            // captured coarsest-grid assembly, factorization and inverse
     cudaStream_t cap_stream = nullptr;  // private stream the graphs are captured on
@@ -209,6 +218,15 @@ int stencil_bf16(const Ctx& c, int mode, const OpLaunch& L, const ModalK<float>&
 // Returns -1 for any other combination, else as stencil().
 int stencil_df(const Ctx& c, int mode, const OpLaunch& L, const ModalK<dfl>& mk, const double* E, const uint8_t* mask,
                const double* u, const double* f, double* out64, float* out32, double* dot_partials);
+// ---- op64.cu: FP64 operators by elements -----------------------------------
+// Levels of at most this many elements take op64_apply for every mode but
+// JACOBI0.
+constexpr long long kOp64Max = 1LL << 20;
+Op64Plan op64_plan(const Geom& g, int nsm);
+// as stencil(); Dinv is read by JACOBI and JACOBI2; scratch: p.scratch() doubles
+int op64_apply(const Ctx& c, int mode, const Geom& g, const Op64Plan& p, const ModalK<double>& mk, const double* E,
+               const uint8_t* mask, const double* u, const double* f, double* out, double omega, double* dot_partials,
+               const double* Dinv, double* pout, const double* beta, double* scratch);
 // ---- tc_op.cu: FP32 operators with the element products on tcgen05 tensor cores
 OpLaunch op_launch(const Geom& g, int ty, int target_ctas, int resident_ctas);
 OpLaunch op_launch_tc(const Geom& g, int nsm);

@@ -85,6 +85,10 @@ int op_apply(topo_grid* h, int mode, int l, const T* u, const T* f, T* out, doub
         if constexpr (std::is_same<T, float>::value)
             np = stencil_tc(h->ctx(), mode, lv.optc, h->mk32->kdiag, lv.E32, lv.mask, u, f, out, (float)h->prm.omega,
                             h->tcB, dot, h->tc_err);
+    } else if (std::is_same<T, double>::value && h->el64 && lv.p64.cz > 0 && mode != ST_JACOBI0) {
+        if constexpr (std::is_same<T, double>::value)
+            np = op64_apply(h->ctx(), mode, lv.g, lv.p64, *h->mk64, lv.E64, lv.mask, u, f, out, h->prm.omega, dot,
+                            lv.Dinv64, pout, beta, h->el64);
     } else {
         np = stencil<T>(h->ctx(), mode, P<T>::op(lv), P<T>::mk(h), P<T>::E(lv), lv.mask, u, f, out,
                         (T)h->prm.omega, dot, P<T>::Dinv(lv), pout, beta);
