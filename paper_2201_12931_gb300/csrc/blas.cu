@@ -11,6 +11,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "fp64.cuh"
 
 namespace topo {
 
@@ -261,60 +262,73 @@ __global__ void k_axpy_f32(long long n, const float* __restrict__ d, double* __r
 // threads, instead of one tile per CTA.
 constexpr int kStrip = 4;
 
-// Cholesky of diagonal block kb by one CTA of 128 threads (right-looking, in
-// shared memory; the pivot by one thread: rs = rsqrt(d), L_jj = d rs), then
-// L_kk^-1 by forward elimination (row j of X = B_j / L_jj, then
-// B_i -= L_ij X_j for the rows below).  L goes back to the block (zeros above
-// the diagonal), L_kk^-1 to Dk (block kb: TB x TB row-major at Dk + kb TB^2).
-// A non-positive or non-finite pivot sets info to its row + 1 (first one
-// wins) and continues with pivot 1.
-__global__ void __launch_bounds__(128) k_potrf_diag(double* __restrict__ A, int npad, int kb, int* info,
+// Cholesky factor of diagonal block kb and its inverse by one CTA, as
+// A = U D U^T (U unit lower) with U^-1 carried along, so that a pivot step is
+// a reciprocal, one rank-one update and one barrier.  16 warps, lane = row:
+// warps 0-7 hold columns w, w + 8, w + 16, w + 24 of A in registers, warps
+// 8-15 those of U^-1.  The chain of 32 pivots bounds it, in latency of FP64
+// instructions (their pipe takes 16 clocks per warp instruction and SM): the
+// columns are published unscaled with 1 / d beside them, and the square
+// roots of the pivots come at the end, all 32 at once: L = U D^(1/2),
+// L^-1 = D^(-1/2) U^-1.  L goes back to the block (zeros above the diagonal),
+// L^-1 to Dk (block kb: TB x TB row-major at Dk + kb TB^2).  A non-positive
+// or non-finite pivot sets info to its row + 1 (first one wins) and continues
+// with pivot 1.
+__global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int npad, int kb, int* info,
                                                     double* __restrict__ Dk) {
-    __shared__ double sA[TB][TB + 1];
-    __shared__ double sX[TB][TB + 1];
-    __shared__ double sR[TB];
-    const int tid = threadIdx.x;
+    __shared__ double col[2][TB], rec[2], piv[TB], root[TB];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, wc = w & 7;
+    const bool isA = w < 8;
     const long long base = (long long)kb * TB;
-    for (int e = tid; e < TB * TB; e += 128) {
-        const int r = e / TB, c = e % TB;
-        sA[r][c] = A[(base + r) * npad + base + c];
-        sX[r][c] = (r == c) ? 1.0 : 0.0;
+    double a[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int c = wc + 8 * s;
+        a[s] = isA ? A[(base + lane) * npad + base + c] : (lane == c ? 1.0 : 0.0);
+    }
+#pragma unroll
+    for (int js = 0; js < 4; ++js)
+        for (int jw = 0; jw < 8; ++jw) {
+            const int j = 8 * js + jw, b = j & 1;
+            if (isA && wc == jw) {
+                double d = __shfl_sync(0xffffffffu, a[js], j);
+                if (!(d > 0.0) || !isfinite(d)) {
+                    if (lane == 0) atomicCAS(info, 0, (int)(base + j) + 1);
+                    d = 1.0;
+                }
+                const double y = seed_range(d) ? recip_seeded(d) : 1.0 / d;
+                col[b][lane] = a[js];
+                if (lane == 0) {
+                    rec[b] = y;
+                    piv[j] = d;
+                }
+            }
+            __syncthreads();
+            const double l = lane > j ? col[b][lane] * rec[b] : 0.0;   // U_ij
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const int c = wc + 8 * s;
+                // (c <= j: A's column is done; c > j: U^-1 has a zero in row j)
+                if (isA ? c > j : c <= j) {
+                    const double r = isA ? col[b][c] : __shfl_sync(0xffffffffu, a[s], j);
+                    a[s] = fma(-l, r, a[s]);
+                }
+            }
+        }
+    if (w == 0) {
+        const double d = piv[lane];   // written by warps that have passed the last barrier
+        root[lane] = rsqrt(d);
     }
     __syncthreads();
-    for (int j = 0; j < TB; ++j) {
-        if (tid == 0) {
-            double d = sA[j][j];
-            if (!(d > 0.0) || !isfinite(d)) {
-                atomicCAS(info, 0, (int)(base + j) + 1);
-                d = 1.0;
-            }
-            const double rs = rsqrt(d);
-            sA[j][j] = d * rs;
-            sR[j] = rs;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int c = wc + 8 * s;
+        if (isA) {
+            const double v = lane == c ? piv[c] : a[s];
+            A[(base + lane) * npad + base + c] = lane >= c ? v * root[c] : 0.0;
+        } else {
+            Dk[base * TB + lane * TB + c] = lane >= c ? a[s] * root[lane] : 0.0;
         }
-        __syncthreads();
-        if (tid > j && tid < TB) sA[tid][j] *= sR[j];
-        __syncthreads();
-        for (int e = (j + 1) * TB + tid; e < TB * TB; e += 128) {   // rows below j only
-            const int i = e / TB, k = e % TB;
-            if (k > j && k <= i) sA[i][k] -= sA[i][j] * sA[k][j];
-        }
-        __syncthreads();
-    }
-    for (int j = 0; j < TB; ++j) {
-        if (tid <= j) sX[j][tid] *= sR[j];
-        __syncthreads();
-        for (int e = (j + 1) * TB + tid; e < TB * TB; e += 128) {   // rows below j only
-            const int i = e / TB, c = e % TB;
-            if (c <= j) sX[i][c] -= sA[i][j] * sX[j][c];
-        }
-        __syncthreads();
-    }
-    double* D = Dk + base * TB;
-    for (int e = tid; e < TB * TB; e += 128) {
-        const int r = e / TB, c = e % TB;
-        A[(base + r) * npad + base + c] = (c <= r) ? sA[r][c] : 0.0;
-        D[e] = sX[r][c];
     }
 }
 
@@ -525,7 +539,7 @@ void chol_factor(const Ctx& c, double* A, int npad, int band, int* info, double*
     const int nb = npad / TB, bb = band_blocks(band);
     cudaMemsetAsync(info, 0, sizeof(int), c.s);
     for (int kb = 0; kb < nb; ++kb) {
-        k_potrf_diag<<<1, 128, 0, c.s>>>(A, npad, kb, info, Dk);
+        k_potrf_diag<<<1, 512, 0, c.s>>>(A, npad, kb, info, Dk);
         TOPO_LAUNCH_CHECK(c);
         const int m = std::min(nb - kb - 1, bb);
         if (m > 0) {
