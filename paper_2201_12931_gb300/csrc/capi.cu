@@ -415,6 +415,10 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
         d.nd = split(a.nd); d.no = split(a.no); d.sc = split(a.sc); d.bp = split(a.bp); d.bq = split(a.bq);
         d.td = split(a.td); d.to = split(a.to); d.cg = split(a.cg); d.kdiag = split(a.kdiag);
     }
+    if (brick_init() != cudaSuccess) {
+        h->err = std::string("operator kernels: ") + cudaGetErrorString(cudaGetLastError());
+        return bail(TOPO_CUDA);
+    }
     h->lev.resize(h->L);
     h->npartials = kRedBlocks;
     int nsm = 0;
@@ -430,6 +434,8 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
         lv.op32 = op_launch32(lv.g, nsm);
         lv.op64 = op_launch64(lv.g, nsm);
         lv.optc = op_launch_tc(lv.g, nsm);
+        lv.brick = lv.g.nn <= kBrickMax;
+        if (lv.brick) h->npartials = std::max(h->npartials, brick_ctas(lv.g));
         if (lv.g.ne <= kOp64Max) lv.p64 = op64_plan(lv.g, nsm);
         h->npartials = std::max(h->npartials, (long long)lv.p64.blocks);
         h->npartials = std::max(h->npartials, std::max(lv.op32.ctas(), std::max(lv.op64.ctas(), lv.optc.ctas())));

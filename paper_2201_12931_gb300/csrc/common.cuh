@@ -68,6 +68,7 @@ struct Level {
     OpLaunch op32, op64;      // operator launch geometry per precision
     OpLaunch optc;            // tensor-core FP32 operator (tc_op.cu)
     Op64Plan p64;             // FP64 operator by elements (op64.cu)
+    bool brick = false;       // FP32 operators by bricks (op_brick.cu)
     double scale = 1.0;       // 2^l
     double* rho = nullptr;    // homogenized density
     double* E64 = nullptr;    // 2^l * (Emin + rho^p (E0 - Emin))
@@ -227,6 +228,16 @@ Op64Plan op64_plan(const Geom& g, int nsm);
 int op64_apply(const Ctx& c, int mode, const Geom& g, const Op64Plan& p, const ModalK<double>& mk, const double* E,
                const uint8_t* mask, const double* u, const double* f, double* out, double omega, double* dot_partials,
                const double* Dinv, double* pout, const double* beta, double* scratch);
+// ---- op_brick.cu: FP32 operators of small levels ---------------------------
+// Levels of at most this many nodes take brick_apply for every mode but JACOBI0.
+constexpr long long kBrickMax = 200000;
+cudaError_t brick_init();   // per device, before the first launch
+long long brick_ctas(const Geom& g);
+// as stencil(); Dinv is read by JACOBI and JACOBI2; ec (JACOBI only, may be
+// null): the iterate is u + P~ ec, ec and its mask maskc on the next coarser level
+int brick_apply(const Ctx& c, int mode, const Geom& g, const ModalK<float>& mk, const float* E, const uint8_t* mask,
+                const float* u, const float* f, float* out, float omega, double* dot_partials, const float* Dinv,
+                float* pout, const double* beta, const float* ec, const uint8_t* maskc);
 // ---- tc_op.cu: FP32 operators with the element products on tcgen05 tensor cores
 OpLaunch op_launch(const Geom& g, int ty, int target_ctas, int resident_ctas);
 OpLaunch op_launch_tc(const Geom& g, int nsm);

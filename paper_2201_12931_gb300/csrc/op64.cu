@@ -138,7 +138,10 @@ __global__ void __launch_bounds__(128) k_node64(const double* __restrict__ scrat
                 }
             }
         const unsigned m = mask[n];
-        const double d = (MODE == ST_JACOBI || MODE == ST_JACOBI2) ? omega * Dinv[n] : 0.0;
+        double d = (MODE == ST_JACOBI || MODE == ST_JACOBI2) ? omega * Dinv[n] : 0.0;
+        // a node without stiffness has no diagonal: the sweep is not finite there
+        if constexpr (MODE == ST_JACOBI)
+            if (__double2hiint(d) == 0) d = __longlong_as_double(0x7ff0000000000000ll);
         const double b = MODE == ST_APPLY_P && beta ? *beta : 0.0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {

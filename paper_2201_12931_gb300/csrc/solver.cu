@@ -54,7 +54,7 @@ struct P<float> {
 
 template <typename T>
 int op_apply(topo_grid* h, int mode, int l, const T* u, const T* f, T* out, double* dot, T* pout,
-             const double* beta) {
+             const double* beta, const T* ec) {
     Level& lv = h->lev[l];
     // FP32 operators with K.u on the tensor cores (the first sweep needs none)
     const bool tc = std::is_same<T, float>::value && h->prm.tensor_cores != 0 &&
@@ -85,6 +85,10 @@ int op_apply(topo_grid* h, int mode, int l, const T* u, const T* f, T* out, doub
         if constexpr (std::is_same<T, float>::value)
             np = stencil_tc(h->ctx(), mode, lv.optc, h->mk32->kdiag, lv.E32, lv.mask, u, f, out, (float)h->prm.omega,
                             h->tcB, dot, h->tc_err);
+    } else if (std::is_same<T, float>::value && lv.brick && mode != ST_JACOBI0) {
+        if constexpr (std::is_same<T, float>::value)
+            np = brick_apply(h->ctx(), mode, lv.g, *h->mk32, lv.E32, lv.mask, u, f, out, (float)h->prm.omega, dot,
+                             lv.Dinv32, pout, beta, ec, ec ? h->lev[l + 1].mask : nullptr);
     } else if (std::is_same<T, double>::value && h->el64 && lv.p64.cz > 0 && mode != ST_JACOBI0) {
         if constexpr (std::is_same<T, double>::value)
             np = op64_apply(h->ctx(), mode, lv.g, lv.p64, *h->mk64, lv.E64, lv.mask, u, f, out, h->prm.omega, dot,
@@ -102,9 +106,16 @@ int op_apply(topo_grid* h, int mode, int l, const T* u, const T* f, T* out, doub
     return dot ? np : 0;
 }
 template int op_apply<double>(topo_grid*, int, int, const double*, const double*, double*, double*, double*,
-                              const double*);
+                              const double*, const double*);
 template int op_apply<float>(topo_grid*, int, int, const float*, const float*, float*, double*, float*,
-                             const double*);
+                             const double*, const float*);
+
+// whether a Jacobi sweep of level l takes the coarse correction along (op_apply's ec)
+template <typename T>
+static bool fuse_prolong(const topo_grid* h, int l) {
+    return std::is_same<T, float>::value && h->lev[l].brick && h->prm.tensor_cores == 0 &&
+           !(h->prm.homogenize == 2 && l > 0);
+}
 
 template <typename T>
 int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot) {
@@ -142,10 +153,12 @@ int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot) {
     VBuf<T>& vc = P<T>::vb(lc);
     restrict_residual<T>(c, lv.g, lv.mask, lc.mask, oth, vc.f);
     vcycle<T>(h, l + 1, vc.f, vc.a, vc.b, nullptr);
-    prolong_add<T>(c, lv.g, lv.mask, lc.mask, vc.a, cur);
+    const T* ec = post > 0 && fuse_prolong<T>(h, l) ? vc.a : nullptr;
+    if (!ec) prolong_add<T>(c, lv.g, lv.mask, lc.mask, vc.a, cur);
     int np = 0;
     for (int s = 0; s < post; ++s) {
-        np = op_apply<T>(h, ST_JACOBI, l, cur, f, oth, (s == post - 1) ? dot : nullptr);
+        np = op_apply<T>(h, ST_JACOBI, l, cur, f, oth, (s == post - 1) ? dot : nullptr, nullptr, nullptr,
+                         s == 0 ? ec : nullptr);
         T* t = cur; cur = oth; oth = t;
     }
     if (post == 0 && dot) {
