@@ -423,18 +423,69 @@ __global__ void k_transpose(const double* __restrict__ W, double* __restrict__ W
     WT[((long long)bx * TB + ty) * npad + (long long)by * TB + tx] = s[tx][ty];
 }
 
-// y_i = sum_{j<=i} W_ij r_j  (lower) or sum_{j>=i} (upper); warp per row
+// y_i = sum_{j<=i} W_ij r_j (lower) or sum_{j>=i} (upper); warp per row.  FP64
+// matrices: FP64 sums.  FP32 matrices: every product and sum with its exact
+// rounding error carried in a second FP32 word (TwoProduct by fused
+// multiply-add, Knuth's TwoSum; the sum is as if accumulated in 48 bits
+// before the one rounding of the result): 9 FP32 instructions per entry
+// where two conversions and an FP64 multiply-add take 48 issue cycles of the
+// SM, which bounded the product (25 us for 1911 rows).
+__device__ __forceinline__ void two_sum_into(float& s, float& c, float p) {
+    const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b)));
+    s = t;
+}
 template <typename T, bool LOWER>
 __global__ void k_trigemv(int n, int npad, const T* __restrict__ M, const T* __restrict__ v, T* __restrict__ y) {
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= n) return;
     const int j0 = LOWER ? 0 : row, j1 = LOWER ? row + 1 : n;
-    double s = 0.0;
     const T* mr = M + (long long)row * npad;
-    for (int j = j0 + lane; j < j1; j += 32) s += (double)mr[j] * (double)v[j];
-    s = warp_sum(s);
-    if (lane == 0) y[row] = (T)s;
+    if constexpr (std::is_same<T, float>::value) {
+        float s[2] = {0.0f, 0.0f}, c[2] = {0.0f, 0.0f};   // two chains
+        auto add = [&](int q, float a, float b) {
+            const float p = __fmul_rn(a, b);
+            c[q] = __fadd_rn(c[q], __fmaf_rn(a, b, -p));
+            two_sum_into(s[q], c[q], p);
+        };
+        int j = j0 + lane;
+        for (; j + 224 < j1; j += 256) {   // eight loads of each in flight
+            float a[8], b[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                a[q] = mr[j + 32 * q];
+                b[q] = v[j + 32 * q];
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) add(q & 1, a[q], b[q]);
+        }
+        for (; j < j1; j += 32) add(0, mr[j], v[j]);
+        c[0] += c[1];
+        two_sum_into(s[0], c[0], s[1]);
+        for (int o = 16; o > 0; o >>= 1) {
+            const float so = __shfl_xor_sync(0xffffffffu, s[0], o), co = __shfl_xor_sync(0xffffffffu, c[0], o);
+            c[0] += co;
+            two_sum_into(s[0], c[0], so);
+        }
+        if (lane == 0) y[row] = s[0] + c[0];
+    } else {
+        double s[2] = {0.0, 0.0};
+        int j = j0 + lane;
+        for (; j + 96 < j1; j += 128) {
+            double a[4], b[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                a[q] = mr[j + 32 * q];
+                b[q] = v[j + 32 * q];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[q & 1] = fma(a[q], b[q], s[q & 1]);
+        }
+        for (; j < j1; j += 32) s[0] = fma(mr[j], v[j], s[0]);
+        const double t = warp_sum(s[0] + s[1]);
+        if (lane == 0) y[row] = t;
+    }
 }
 
 }  // namespace
@@ -577,10 +628,10 @@ void transpose_dense(const Ctx& c, const double* W, double* WT, int npad) {
 
 template <typename T>
 void coarse_apply(const Ctx& c, int n, int npad, const T* W, const T* WT, const T* rhs, T* y, T* out) {
-    const unsigned blocks = (unsigned)((n + 7) / 8);
-    k_trigemv<T, true><<<blocks, 256, 0, c.s>>>(n, npad, W, rhs, y);
+    const unsigned blocks = (unsigned)((n + 3) / 4);   // four rows a block: small grids on all SMs
+    k_trigemv<T, true><<<blocks, 128, 0, c.s>>>(n, npad, W, rhs, y);
     TOPO_LAUNCH_CHECK(c);
-    k_trigemv<T, false><<<blocks, 256, 0, c.s>>>(n, npad, WT, y, out);
+    k_trigemv<T, false><<<blocks, 128, 0, c.s>>>(n, npad, WT, y, out);
     TOPO_LAUNCH_CHECK(c);
 }
 template void coarse_apply<double>(const Ctx&, int, int, const double*, const double*, const double*, double*,
