@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "fp64.cuh"
+#include "tail.cuh"
 
 namespace topo {
 
@@ -66,33 +67,11 @@ __global__ void __launch_bounds__(1024) k_reduce_to(const double* __restrict__ p
     if (threadIdx.x == 0) *dst = s;
 }
 
-__global__ void __launch_bounds__(1024) k_cg_alpha(const double* __restrict__ p, int n, Scalars* sc,
-                                                   double* __restrict__ hist) {
+__global__ void __launch_bounds__(1024) k_cg_scalar(int kind, const double* __restrict__ p, int n, Scalars* sc,
+                                                    double* __restrict__ hist) {
     __shared__ double sh[32];
-    const double pq = sum_partials(p, n, sh);
-    if (threadIdx.x == 0) {
-        sc->pq = pq;
-        if (pq > 0.0 && isfinite(pq) && isfinite(sc->rz)) {
-            sc->alpha = sc->rz / pq;
-        } else {
-            sc->alpha = 0.0;
-            sc->aux = 1.0;   // breakdown flag, read by the host
-        }
-        if (hist) *hist = sc->alpha;
-    }
-}
-
-__global__ void __launch_bounds__(1024) k_cg_beta(const double* __restrict__ p, int n, Scalars* sc) {
-    __shared__ double sh[32];
-    const double rz = sum_partials(p, n, sh);
-    if (threadIdx.x == 0) {
-        const double old = sc->rz;
-        sc->rz_old = old;
-        sc->rz_new = rz;
-        sc->beta = (old != 0.0 && isfinite(rz)) ? rz / old : 0.0;
-        if (!isfinite(rz)) sc->aux = 1.0;
-        sc->rz = rz;
-    }
+    const double s = sum_partials(p, n, sh);
+    if (threadIdx.x == 0) cg_scalar(kind, s, sc, hist);
 }
 
 __global__ void __launch_bounds__(1024) k_cg_beta_flexible(const double* __restrict__ p, int n, Scalars* sc) {
@@ -151,10 +130,11 @@ __global__ void __launch_bounds__(256) k_update_xr(long long n, const Scalars* _
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
-// r -= alpha q and per-block partial sums of r.r (as k_update_xr without x)
+// r -= alpha q and r.r (as k_update_xr without x; the last block reduces)
 template <typename T>
-__global__ void __launch_bounds__(256) k_update_r(long long n, const Scalars* __restrict__ sc, const T* __restrict__ q,
-                                                  T* __restrict__ r, double* __restrict__ partials) {
+__global__ void __launch_bounds__(256) k_update_r(long long n, const Scalars* sc, const T* __restrict__ q,
+                                                  T* __restrict__ r, double* __restrict__ partials,
+                                                  const DotTail tail) {
     __shared__ double sh[32];
     const T a = (T)sc->alpha;
     double s = 0.0;
@@ -184,6 +164,7 @@ __global__ void __launch_bounds__(256) k_update_r(long long n, const Scalars* __
     }
     s = block_sum(s, sh);
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    dot_tail<256>(tail, partials, gridDim.x, threadIdx.x);
 }
 
 // x += alpha_j p_j, j = 0 .. count-1 in order: per entry the same fused
@@ -504,11 +485,11 @@ void reduce_to(const Ctx& c, const double* partials, int n, double* dst) {
     TOPO_LAUNCH_CHECK(c);
 }
 void cg_alpha(const Ctx& c, const double* partials, int n, Scalars* sc, double* hist) {
-    k_cg_alpha<<<1, 1024, 0, c.s>>>(partials, n, sc, hist);
+    k_cg_scalar<<<1, 1024, 0, c.s>>>(TAIL_ALPHA, partials, n, sc, hist);
     TOPO_LAUNCH_CHECK(c);
 }
 void cg_beta(const Ctx& c, const double* partials, int n, Scalars* sc) {
-    k_cg_beta<<<1, 1024, 0, c.s>>>(partials, n, sc);
+    k_cg_scalar<<<1, 1024, 0, c.s>>>(TAIL_BETA, partials, n, sc, nullptr);
     TOPO_LAUNCH_CHECK(c);
 }
 void cg_beta_flexible(const Ctx& c, const double* partials, int n, Scalars* sc) {
@@ -536,12 +517,14 @@ template void cg_update_p<double>(const Ctx&, long long, const Scalars*, const d
 template void cg_update_p<float>(const Ctx&, long long, const Scalars*, const float*, float*);
 
 template <typename T>
-void cg_update_r(const Ctx& c, long long n, const Scalars* sc, const T* q, T* r, double* partials) {
-    k_update_r<T><<<kRedBlocks, 256, 0, c.s>>>(n, sc, q, r, partials);
+void cg_update_r(const Ctx& c, long long n, Scalars* sc, const T* q, T* r, double* partials, unsigned* ticket) {
+    const unsigned g = grid_for(n, 1024);   // four entries per thread until the GPU is full
+    k_update_r<T><<<g > kUpdateBlocks ? kUpdateBlocks : g, 256, 0, c.s>>>(n, sc, q, r, partials,
+                                                                       DotTail{TAIL_RR, sc, nullptr, ticket});
     TOPO_LAUNCH_CHECK(c);
 }
-template void cg_update_r<double>(const Ctx&, long long, const Scalars*, const double*, double*, double*);
-template void cg_update_r<float>(const Ctx&, long long, const Scalars*, const float*, float*, double*);
+template void cg_update_r<double>(const Ctx&, long long, Scalars*, const double*, double*, double*, unsigned*);
+template void cg_update_r<float>(const Ctx&, long long, Scalars*, const float*, float*, double*, unsigned*);
 
 template <typename T>
 void cg_flush_x(const Ctx& c, long long n, T* const* ring, const double* alpha, int count, T* x) {

@@ -170,7 +170,7 @@ void free_all(topo_grid* h) {
     F(h->cs.A); F(h->cs.W64); F(h->cs.WT64); F(h->cs.W32); F(h->cs.WT32); F(h->cs.y64); F(h->cs.y32);
     F(h->cs.info); F(h->cs.Dk);
     F(h->x); F(h->f); F(h->r); F(h->z); F(h->p); F(h->q);
-    F(h->r32); F(h->z32); F(h->p32); F(h->q32); F(h->d32); F(h->alpha_hist); F(h->el64);
+    F(h->r32); F(h->z32); F(h->p32); F(h->q32); F(h->d32); F(h->alpha_hist); F(h->ticket); F(h->el64);
     for (auto& d : h->dring64) F(d);
     for (auto& d : h->dring32) F(d);
     F(h->K0d); F(h->K0f);
@@ -420,7 +420,7 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
         return bail(TOPO_CUDA);
     }
     h->lev.resize(h->L);
-    h->npartials = kRedBlocks;
+    h->npartials = std::max(kRedBlocks, kUpdateBlocks);
     int nsm = 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || nsm <= 0) {
         cudaGetLastError();
@@ -474,6 +474,7 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
     TRY(dalloc(h, &h->partials, (size_t)h->npartials));
     TRY(dalloc(h, &h->sc, 1));
     TRY(dalloc(h, &h->alpha_hist, kDirRing));
+    TRY(dalloc(h, &h->ticket, 1));
     h->cs.n = (int)std::min<long long>(3 * h->lev[h->L - 1].g.nn, 1LL << 30);
     h->cs.npad = (h->cs.n + 31) / 32 * 32;
     TRY(alloc_precision(h, p.precision == TOPO_FP64));
@@ -495,6 +496,7 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
               cudaMemsetAsync(h->sc, 0, sizeof(Scalars), h->stream) == cudaSuccess &&
               cudaMemsetAsync(h->dflag, 0, sizeof(int), h->stream) == cudaSuccess &&
               cudaMemsetAsync(h->tc_err, 0, sizeof(int), h->stream) == cudaSuccess &&
+              cudaMemsetAsync(h->ticket, 0, sizeof(unsigned), h->stream) == cudaSuccess &&
               cudaMemcpyAsync(h->tcB, tcimg.data(), sizeof(uint32_t) * kTcBWords, cudaMemcpyHostToDevice,
                               h->stream) == cudaSuccess;
     for (auto& lv : h->lev) ok = ok && cudaMemsetAsync(lv.mask, 0, lv.g.nn, h->stream) == cudaSuccess;

@@ -119,6 +119,15 @@ struct Scalars {              // device-resident CG scalars
     double rz_old;            // z.r of the previous iteration (flexible beta)
 };
 
+// What the last block of a kernel with partial sums does with them (tail.cuh)
+enum TailKind { TAIL_NONE, TAIL_ALPHA, TAIL_BETA, TAIL_RR };
+struct DotTail {
+    int kind = TAIL_NONE;
+    Scalars* sc = nullptr;
+    double* hist = nullptr;       // TAIL_ALPHA: alpha of the direction's ring slot, may be null
+    unsigned* ticket = nullptr;   // device counter, 0 between kernels
+};
+
 }  // namespace topo
 
 struct topo_grid {
@@ -173,6 +182,7 @@ struct topo_grid {
     double* dring64[topo::kDirRing - 2] = {};
     float* dring32[topo::kDirRing - 2] = {};
     double* alpha_hist = nullptr;   // device: alpha of each ring slot
+    unsigned* ticket = nullptr;     // device: blocks that have finished (DotTail)
     double* el64 = nullptr;         // face contributions of the FP64 operator by elements (op64.cu)
     topo::PcgGraph graph64[topo::kDirRing], graph32[topo::kDirRing];   // captured PCG iterations per ring slot
     topo::PcgGraph coarse_graph;            // captured coarsest-grid assembly, factorization and inverse
@@ -184,6 +194,7 @@ struct topo_grid {
 
 namespace topo {
 
+constexpr int kUpdateBlocks = 8 * 152;   // largest grid of cg_update_r: 2048 threads on every SM
 constexpr int kRedBlocks = 1024;   // fixed grid of reduction kernels (deterministic order)
 constexpr int kProfMax = 65536;    // launch records of topo_profile_enable
 
@@ -227,7 +238,7 @@ Op64Plan op64_plan(const Geom& g, int nsm);
 // as stencil(); Dinv is read by JACOBI and JACOBI2; scratch: p.scratch() doubles
 int op64_apply(const Ctx& c, int mode, const Geom& g, const Op64Plan& p, const ModalK<double>& mk, const double* E,
                const uint8_t* mask, const double* u, const double* f, double* out, double omega, double* dot_partials,
-               const double* Dinv, double* pout, const double* beta, double* scratch);
+               const double* Dinv, double* pout, const double* beta, double* scratch, const DotTail& tail);
 // ---- op_brick.cu: FP32 operators of small levels ---------------------------
 // Levels of at most this many nodes take brick_apply for every mode but JACOBI0.
 constexpr long long kBrickMax = 200000;
@@ -237,7 +248,7 @@ long long brick_ctas(const Geom& g);
 // null): the iterate is u + P~ ec, ec and its mask maskc on the next coarser level
 int brick_apply(const Ctx& c, int mode, const Geom& g, const ModalK<float>& mk, const float* E, const uint8_t* mask,
                 const float* u, const float* f, float* out, float omega, double* dot_partials, const float* Dinv,
-                float* pout, const double* beta, const float* ec, const uint8_t* maskc);
+                float* pout, const double* beta, const float* ec, const uint8_t* maskc, const DotTail& tail);
 // ---- tc_op.cu: FP32 operators with the element products on tcgen05 tensor cores
 OpLaunch op_launch(const Geom& g, int ty, int target_ctas, int resident_ctas);
 OpLaunch op_launch_tc(const Geom& g, int nsm);
@@ -310,9 +321,9 @@ void cg_update_xr(const Ctx& c, long long n, const Scalars* sc, const T* p, cons
                   double* partials);
 template <typename T>
 void cg_update_p(const Ctx& c, long long n, const Scalars* sc, const T* z, T* p);
-// r -= alpha q with partial sums of r.r (x updated later by cg_flush_x)
+// r -= alpha q and sc->rr = r.r (x updated later by cg_flush_x)
 template <typename T>
-void cg_update_r(const Ctx& c, long long n, const Scalars* sc, const T* q, T* r, double* partials);
+void cg_update_r(const Ctx& c, long long n, Scalars* sc, const T* q, T* r, double* partials, unsigned* ticket);
 // x += alpha_j p_j for j = 0 .. count-1 in that order (the same operations as
 // count successive x += alpha p steps); p_j = ring[j], alpha_j = alpha[j]
 template <typename T>

@@ -19,6 +19,7 @@
 
 #include "common.cuh"
 #include "operator.cuh"
+#include "tail.cuh"
 
 namespace topo {
 
@@ -108,7 +109,8 @@ __global__ void __launch_bounds__(128) k_node64(const double* __restrict__ scrat
                                                 const double* __restrict__ u, const double* __restrict__ f,
                                                 const double* __restrict__ Dinv, double* __restrict__ out, int nx,
                                                 int ny, int nz, int cz, double omega, double* __restrict__ partials,
-                                                double* __restrict__ pout, const double* __restrict__ beta) {
+                                                double* __restrict__ pout, const double* __restrict__ beta,
+                                                const DotTail tail) {
     __shared__ double sred[4];
     const int NX = nx + 1, NY = ny + 1, nn = NX * NY * (nz + 1);
     const int ncol = nx * ny, nt = ncol * ((nz + cz - 1) / cz);
@@ -174,6 +176,7 @@ __global__ void __launch_bounds__(128) k_node64(const double* __restrict__ scrat
         if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = dot;
         __syncthreads();
         if (threadIdx.x == 0) partials[blockIdx.x] = (sred[0] + sred[1]) + (sred[2] + sred[3]);
+        dot_tail<128>(tail, partials, gridDim.x, threadIdx.x);
     }
 }
 
@@ -201,13 +204,13 @@ Op64Plan op64_plan(const Geom& g, int nsm) {
 
 int op64_apply(const Ctx& c, int mode, const Geom& g, const Op64Plan& p, const ModalK<double>& mk, const double* E,
                const uint8_t* mask, const double* u, const double* f, double* out, double omega, double* dot,
-               const double* Dinv, double* pout, const double* beta, double* scratch) {
+               const double* Dinv, double* pout, const double* beta, double* scratch, const DotTail& tail) {
     const unsigned ge = (unsigned)((p.nt + 31) / 32), gn = (unsigned)p.blocks;
 #define EL(IN) \
     k_el64<IN><<<ge, 32, 0, c.s>>>(mk, E, mask, u, f, Dinv, g.nx, g.ny, g.nz, p.cz, omega, beta, scratch)
 #define ND(MODE, DOT)                                                                                               \
     k_node64<MODE, DOT><<<gn, 128, 0, c.s>>>(scratch, mask, u, f, Dinv, out, g.nx, g.ny, g.nz, p.cz, omega, dot, pout, \
-                                             beta)
+                                             beta, tail)
     if (mode == ST_APPLY_P) EL(IN_P);
     else if (mode == ST_JACOBI2) EL(IN_F);
     else EL(IN_U);
@@ -234,7 +237,7 @@ int op64_apply(const Ctx& c, int mode, const Geom& g, const Op64Plan& p, const M
     TOPO_LAUNCH_CHECK(c);
 #undef EL
 #undef ND
-    return mode == ST_JACOBI2 ? 0 : p.blocks;
+    return mode == ST_JACOBI2 || !dot ? 0 : (tail.kind != TAIL_NONE ? -1 : p.blocks);
 }
 
 }  // namespace topo

@@ -12,12 +12,11 @@
 // arithmetic that an idle GPU has to spare and is why large grids keep the
 // z-march (shared memory traffic: 16 128-bit accesses per element here).
 // The correction of the coarse grid can be added while loading, which saves
-// the prolongation's launch and its pass over the iterate.  Measured: state
-// step on 64x32x32 elements (4 levels) 16.8 -> 14.0 ms, V-cycle on 128x64x64
-// (whose coarse levels these are) 305 -> 273 us.
+// the prolongation's launch and its pass over the iterate.
 #include "common.cuh"
 #include "operator.cuh"
 #include "opio.cuh"
+#include "tail.cuh"
 
 namespace topo {
 
@@ -67,7 +66,7 @@ __global__ void __launch_bounds__(kThreads) k_brick(const ModalK<float> mk, cons
                                                     const int ny, const int nz, const float omega,
                                                     double* __restrict__ partials, float* __restrict__ pout,
                                                     const double* __restrict__ beta, const float* __restrict__ Dinv,
-                                                    const Coarser cr) {
+                                                    const Coarser cr, const DotTail tail) {
     extern __shared__ float4 smem[];
     float4* const val = smem;                 // node values, 0 at fixed DOFs and outside the grid
     float4* const con = smem + kNodes;        // con[a * kElems + e]: contribution of element e to its corner a
@@ -190,6 +189,7 @@ __global__ void __launch_bounds__(kThreads) k_brick(const ModalK<float> mk, cons
             for (int w = 0; w < kThreads / 32; ++w) s += sred[w];
             partials[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = s;
         }
+        dot_tail<kThreads>(tail, partials, gridDim.x * gridDim.y * gridDim.z, tid);
     }
 }
 
@@ -200,9 +200,9 @@ dim3 brick_grid(const Geom& g) {
 template <int MODE, bool DOT, bool PROLONG>
 void launch(const Ctx& c, const Geom& g, const ModalK<float>& mk, const float* E, const uint8_t* mask, const float* u,
             const float* f, float* out, float omega, double* dot, const float* Dinv, float* pout, const double* beta,
-            const Coarser& cr) {
+            const Coarser& cr, const DotTail& tail) {
     k_brick<MODE, DOT, PROLONG><<<brick_grid(g), kThreads, kSmem, c.s>>>(mk, E, mask, u, f, out, g.nx, g.ny, g.nz, omega,
-                                                                       dot, pout, beta, Dinv, cr);
+                                                                       dot, pout, beta, Dinv, cr, tail);
     TOPO_LAUNCH_CHECK(c);
 }
 
@@ -234,9 +234,9 @@ long long brick_ctas(const Geom& g) {
 
 int brick_apply(const Ctx& c, int mode, const Geom& g, const ModalK<float>& mk, const float* E, const uint8_t* mask,
                 const float* u, const float* f, float* out, float omega, double* dot, const float* Dinv, float* pout,
-                const double* beta, const float* ec, const uint8_t* maskc) {
+                const double* beta, const float* ec, const uint8_t* maskc, const DotTail& tail) {
     const Coarser cr{ec, maskc};
-#define GO(MODE, DOT, PRO) launch<MODE, DOT, PRO>(c, g, mk, E, mask, u, f, out, omega, dot, Dinv, pout, beta, cr)
+#define GO(MODE, DOT, PRO) launch<MODE, DOT, PRO>(c, g, mk, E, mask, u, f, out, omega, dot, Dinv, pout, beta, cr, tail)
     switch (mode) {
         case ST_APPLY_P:
             if (dot) GO(ST_APPLY_P, true, false);
@@ -259,7 +259,7 @@ int brick_apply(const Ctx& c, int mode, const Geom& g, const ModalK<float>& mk, 
             break;
     }
 #undef GO
-    return dot ? (int)brick_ctas(g) : 0;
+    return dot ? (tail.kind != TAIL_NONE ? -1 : (int)brick_ctas(g)) : 0;
 }
 
 }  // namespace topo

@@ -54,7 +54,7 @@ struct P<float> {
 
 template <typename T>
 int op_apply(topo_grid* h, int mode, int l, const T* u, const T* f, T* out, double* dot, T* pout,
-             const double* beta, const T* ec) {
+             const double* beta, const T* ec, const DotTail& tail) {
     Level& lv = h->lev[l];
     // FP32 operators with K.u on the tensor cores (the first sweep needs none)
     const bool tc = std::is_same<T, float>::value && h->prm.tensor_cores != 0 &&
@@ -88,11 +88,11 @@ int op_apply(topo_grid* h, int mode, int l, const T* u, const T* f, T* out, doub
     } else if (std::is_same<T, float>::value && lv.brick && mode != ST_JACOBI0) {
         if constexpr (std::is_same<T, float>::value)
             np = brick_apply(h->ctx(), mode, lv.g, *h->mk32, lv.E32, lv.mask, u, f, out, (float)h->prm.omega, dot,
-                             lv.Dinv32, pout, beta, ec, ec ? h->lev[l + 1].mask : nullptr);
+                             lv.Dinv32, pout, beta, ec, ec ? h->lev[l + 1].mask : nullptr, tail);
     } else if (std::is_same<T, double>::value && h->el64 && lv.p64.cz > 0 && mode != ST_JACOBI0) {
         if constexpr (std::is_same<T, double>::value)
             np = op64_apply(h->ctx(), mode, lv.g, lv.p64, *h->mk64, lv.E64, lv.mask, u, f, out, h->prm.omega, dot,
-                            lv.Dinv64, pout, beta, h->el64);
+                            lv.Dinv64, pout, beta, h->el64, tail);
     } else {
         np = stencil<T>(h->ctx(), mode, P<T>::op(lv), P<T>::mk(h), P<T>::E(lv), lv.mask, u, f, out,
                         (T)h->prm.omega, dot, P<T>::Dinv(lv), pout, beta);
@@ -106,9 +106,9 @@ int op_apply(topo_grid* h, int mode, int l, const T* u, const T* f, T* out, doub
     return dot ? np : 0;
 }
 template int op_apply<double>(topo_grid*, int, int, const double*, const double*, double*, double*, double*,
-                              const double*, const double*);
+                              const double*, const double*, const DotTail&);
 template int op_apply<float>(topo_grid*, int, int, const float*, const float*, float*, double*, float*,
-                             const double*, const float*);
+                             const double*, const float*, const DotTail&);
 
 // whether a Jacobi sweep of level l takes the coarse correction along (op_apply's ec)
 template <typename T>
@@ -118,7 +118,7 @@ static bool fuse_prolong(const topo_grid* h, int l) {
 }
 
 template <typename T>
-int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot) {
+int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot, const DotTail& tail) {
     const Ctx c = h->ctx();
     Level& lv = h->lev[l];
     if (l == h->L - 1) {
@@ -158,7 +158,7 @@ int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot) {
     int np = 0;
     for (int s = 0; s < post; ++s) {
         np = op_apply<T>(h, ST_JACOBI, l, cur, f, oth, (s == post - 1) ? dot : nullptr, nullptr, nullptr,
-                         s == 0 ? ec : nullptr);
+                         s == 0 ? ec : nullptr, s == post - 1 ? tail : DotTail());
         T* t = cur; cur = oth; oth = t;
     }
     if (post == 0 && dot) {
@@ -167,8 +167,8 @@ int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot) {
     }
     return dot ? np : 0;
 }
-template int vcycle<double>(topo_grid*, int, const double*, double*, double*, double*);
-template int vcycle<float>(topo_grid*, int, const float*, float*, float*, double*);
+template int vcycle<double>(topo_grid*, int, const double*, double*, double*, double*, const DotTail&);
+template int vcycle<float>(topo_grid*, int, const float*, float*, float*, double*, const DotTail&);
 
 // operator launch with BF16 iterates; level-0 launches are recorded for
 // topo_profile_read (precision slot 2)
@@ -334,7 +334,7 @@ static int pcg_core(topo_grid* h, T* x, T* r, T* z, T* p, T* q, double rr0, doub
                 return vcycle_bf16(h, 0, reinterpret_cast<const float*>(r), reinterpret_cast<float*>(z),
                                    h->partials);
         }
-        return vcycle<T>(h, 0, r, z, vb.a, h->partials);
+        return vcycle<T>(h, 0, r, z, vb.a, h->partials, DotTail{TAIL_BETA, h->sc, nullptr, h->ticket});
     };
     const bool flexible = std::is_same<T, float>::value && h->prm.precision == TOPO_MIXED_BF16;
     // The direction update p = z + beta p is fused into the K.p kernel
@@ -351,7 +351,7 @@ static int pcg_core(topo_grid* h, T* x, T* r, T* z, T* p, T* q, double rr0, doub
     ring[1] = vb.b;   // vb.b of level 0 is free during the solve
     for (int j = 2; j < R; ++j) ring[j] = P<T>::dring(h)[j - 2];
     int np = precond();
-    cg_beta(c, h->partials, np, h->sc);   // sets rz (beta unused on the first step)
+    if (np >= 0) cg_beta(c, h->partials, np, h->sc);   // sets rz (beta unused on the first step)
     if (!fused) cudaMemcpyAsync(p, z, sizeof(T) * n, cudaMemcpyDeviceToDevice, h->stream);
     // step k: K p, alpha, r -= alpha q, r.r, and x += alpha p (per step, or
     // per full ring when fused) on the stream current in h; first step (k = 0):
@@ -362,22 +362,23 @@ static int pcg_core(topo_grid* h, T* x, T* r, T* z, T* p, T* q, double rr0, doub
             const int s = k % R;
             // (the first step reads z in place of p_old: beta is absent, nothing is added)
             const int npa = op_apply<T>(h, ST_APPLY_P, 0, z, k == 0 ? z : ring[(s + R - 1) % R], q, h->partials,
-                                        ring[s], k == 0 ? nullptr : &h->sc->beta);
-            cg_alpha(cc, h->partials, npa, h->sc, h->alpha_hist + s);
-            cg_update_r<T>(cc, n, h->sc, q, r, h->partials);
+                                        ring[s], k == 0 ? nullptr : &h->sc->beta, nullptr,
+                                        DotTail{TAIL_ALPHA, h->sc, h->alpha_hist + s, h->ticket});
+            if (npa >= 0) cg_alpha(cc, h->partials, npa, h->sc, h->alpha_hist + s);
+            cg_update_r<T>(cc, n, h->sc, q, r, h->partials, h->ticket);
             if (s == R - 1) cg_flush_x<T>(cc, n, ring, h->alpha_hist, R, x);
         } else {
             const int npa = op_apply<T>(h, ST_APPLY, 0, p, nullptr, q, h->partials);
             cg_alpha(cc, h->partials, npa, h->sc);
             cg_update_xr<T>(cc, n, h->sc, p, q, x, r, h->partials);
+            reduce_to(cc, h->partials, kRedBlocks, &h->sc->rr);
         }
-        reduce_to(cc, h->partials, kRedBlocks, &h->sc->rr);
     };
     // z = M^-1 r, beta, p = z + beta p, then K p ... (step k)
     auto step_ba = [&](int k) {
         const Ctx cc = h->ctx();
         const int npb = precond();
-        cg_beta(cc, h->partials, npb, h->sc);
+        if (npb >= 0) cg_beta(cc, h->partials, npb, h->sc);
         if (flexible) {   // BF16 rounding makes M^-1 vary slightly between applications
             dot_partials<T, T>(cc, n, z, q, h->partials);
             cg_beta_flexible(cc, h->partials, kRedBlocks, h->sc);

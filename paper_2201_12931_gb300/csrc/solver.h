@@ -5,13 +5,14 @@
 #include "common.cuh"
 
 namespace topo {
-// returns the number of dot partials written (0 without dot); ec (JACOBI on
-// levels that fuse_prolong): the iterate is u + P~ ec, ec on level l + 1
+// returns the number of dot partials written (0 without dot, -1: reduced and
+// the tail done); ec (JACOBI on levels that fuse_prolong): the iterate is
+// u + P~ ec, ec on level l + 1
 template <typename T>
 int op_apply(topo_grid* h, int mode, int l, const T* u, const T* f, T* out, double* dot, T* pout = nullptr,
-             const double* beta = nullptr, const T* ec = nullptr);
+             const double* beta = nullptr, const T* ec = nullptr, const DotTail& tail = DotTail());
 template <typename T>
-int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot);
+int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot, const DotTail& tail = DotTail());
 // V-cycle with BF16 iterates on levels 0 .. L-2 (FP32 arithmetic, FP32
 // right-hand sides and residuals, FP32 coarsest solve); the level-0 result
 // is written in FP32 to out.  f and out are level-0 FP32 vectors distinct

@@ -436,8 +436,7 @@ void launch_op(const Ctx& c, const OpLaunch& L, const ModalK<T>& mk, const typen
                              (int)op_smem_bytes<T>());
         attr = true;
     }
-    k_op<T, TU, TO, MODE, DOT><<<dim3(L.gx, L.gy, L.gz), dim3(kOpTX, op_ty<T>()), op_smem_bytes<T>(), c.s>>>(
-        mk, E, mask, u, f, out, L.g.nx, L.g.ny, L.g.nz, L.cz, omega, dot, pout, beta, Dinv);
+    k_op<T, TU, TO, MODE, DOT><<<dim3(L.gx, L.gy, L.gz), dim3(kOpTX, op_ty<T>()), op_smem_bytes<T>(), c.s>>>(mk, E, mask, u, f, out, L.g.nx, L.g.ny, L.g.nz, L.cz, omega, dot, pout, beta, Dinv);
     TOPO_LAUNCH_CHECK(c);
 }
 

@@ -34,24 +34,29 @@ __global__ void __launch_bounds__(256) k_restrict_z(const uint8_t* __restrict__ 
     if (I >= NXc || J >= NYc) return;
     const int K0 = blockIdx.z * czc, K1 = min(K0 + czc, NZc);
     const long long fplane = (long long)NXf * NYf;
+    // the nine values and masks of a plane are loaded before any is used (a
+    // value is not loaded behind its mask): on small levels the launch is as
+    // long as its chain of loads
     auto plane_sum = [&](int k, T* s) {
         s[0] = s[1] = s[2] = T(0);
         if (k < 0 || k > nzf) return;
+        T v[9][3];
+        unsigned m[9];
 #pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int j = 2 * J + dy;
-            if (j < 0 || j >= NYf) continue;
+        for (int q = 0; q < 9; ++q) {
+            const int i = 2 * I + q % 3 - 1, j = 2 * J + q / 3 - 1;
+            const bool ok = i >= 0 && i < NXf && j >= 0 && j < NYf;
+            const long long n = ok ? i + (long long)NXf * j + fplane * k : 0;
+            m[q] = ok ? maskf[n] : 7u;
 #pragma unroll
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int i = 2 * I + dx;
-                if (i < 0 || i >= NXf) continue;
-                const T w = (dx ? T(0.5) : T(1)) * (dy ? T(0.5) : T(1));
-                const long long n = i + (long long)NXf * j + fplane * k;
-                const unsigned mf = maskf[n];
+            for (int c = 0; c < 3; ++c) v[q][c] = rf[3 * n + c];
+        }
 #pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    if (!((mf >> c) & 1u)) s[c] += w * rf[3 * n + c];
-            }
+        for (int q = 0; q < 9; ++q) {
+            const T w = (q % 3 != 1 ? T(0.5) : T(1)) * (q / 3 != 1 ? T(0.5) : T(1));
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                if (!((m[q] >> c) & 1u)) s[c] += w * v[q][c];
         }
     };
     T lo[3], mid[3], hi[3];
