@@ -182,16 +182,20 @@ __global__ void __launch_bounds__(128) k_node64(const double* __restrict__ scrat
 
 }  // namespace
 
-// Layers per thread: the FP64 instructions of the fullest SM (16 clocks per
-// warp instruction and SM) of both kernels.  A thread of cz layers costs
-// 48 (cz + 1) + 80 cz + 12 (cz - 1) of them, a node 9 + 12 / cz + 6.
+// Layers per thread: the time of the fullest scheduler in both kernels.  Each of
+// the four schedulers of an SM takes 64 clocks per FP64 warp instruction (half
+// a lane per clock; a lone warp measured 78), so a grid wants at least four
+// warps per SM: 48x24x24 elements in 144 warps of 6 layers took 36 us.  A
+// thread of cz layers costs 48 (cz + 1) + 80 cz + 12 (cz - 1) instructions, a
+// node 15 + 12 / cz.
 Op64Plan op64_plan(const Geom& g, int nsm) {
     Op64Plan p;
     double best = -1.0;
+    const long long units = 4ll * nsm;
     for (int cz = 1; cz <= 8 && cz <= g.nz; ++cz) {
         const long long warps = ((long long)g.nx * g.ny * ((g.nz + cz - 1) / cz) + 31) / 32;
-        const double el = (double)((warps + nsm - 1) / nsm) * (48.0 * (cz + 1) + 80.0 * cz + 12.0 * (cz - 1));
-        const double nd = (double)((g.nn + 32ll * nsm - 1) / (32ll * nsm)) * (15.0 + 12.0 / cz);
+        const double el = (double)((warps + units - 1) / units) * (48.0 * (cz + 1) + 80.0 * cz + 12.0 * (cz - 1));
+        const double nd = (double)((g.nn + 32 * units - 1) / (32 * units)) * (15.0 + 12.0 / cz);
         if (best < 0.0 || el + nd < best) {
             best = el + nd;
             p.cz = cz;
