@@ -16,8 +16,8 @@
 // r = 6.  S_e depends only on the distances to the six faces, so it is a
 // table of (2R + 1)^3 entries, with reciprocals for the division.
 //
-// Measured, forward + transpose of 256x128x128 elements: r = 3, 2147 -> 784
-// us; the first call with a new radius 3689 -> 832 us.
+// Measured, forward + transpose of 256x128x128 elements: r = 3, 2149 -> 725
+// us; the first call with a new radius 3690 -> 775 us.
 #include <math.h>
 
 #include "common.cuh"
@@ -118,6 +118,12 @@ __global__ void __launch_bounds__(128) k_filter(const __grid_constant__ FilterW 
         if constexpr (MODE == 1) cxy[l] = ok ? face_class(gj, ny, R) * nc + face_class(gi, nx, R) : 0;
         raw[l] = 0.0;
     }
+    // H^T of a block whose values all have the same weight sum: one division
+    // per output instead of one per staged value (2.25 of them at R = 2)
+    bool uniform = false;
+    if constexpr (MODE == 1)
+        uniform = in && i0 >= 2 * R && i0 + TX + 2 * R <= nx && j0 >= 2 * R && j0 + TY + 2 * R <= ny && k0 >= 2 * R &&
+                  k1 + 2 * R <= nz;
     auto fetch = [&](int k) {
 #pragma unroll
         for (int l = 0; l < NL; ++l)
@@ -144,7 +150,7 @@ __global__ void __launch_bounds__(128) k_filter(const __grid_constant__ FilterW 
                     double t = raw[l];
                     if constexpr (MODE == 1) {
                         const int ct = face_class(k, nz, R) * nc * nc + cxy[l];
-                        if (off[l] >= 0) t = in ? div_by(t, stab[ct], stab[kFilterTab + ct]) : stab[kFilterTab + ct];
+                        if (off[l] >= 0 && !uniform) t = in ? div_by(t, stab[ct], stab[kFilterTab + ct]) : stab[kFilterTab + ct];
                     }
                     if constexpr (MODE == 2)
                         if (off[l] >= 0) t *= raw2[l];
@@ -209,6 +215,9 @@ __global__ void __launch_bounds__(128) k_filter(const __grid_constant__ FilterW 
                 const int ct = face_class(ko, nz, R) * nc * nc + ccol;
                 o = div_by(o, stab[ct], stab[kFilterTab + ct]);
                 if constexpr (MODE == 2) o = o / fmax(gamma, rho[e]);
+            } else if (uniform) {
+                constexpr int ct = (nc * nc + nc + 1) * R;
+                o = div_by(o, stab[ct], stab[kFilterTab + ct]);
             }
             out[e] = o;
         }
@@ -268,8 +277,8 @@ void filter_plan(const Geom& g, double r, int nsm, FilterPlan* p) {
     for (int tx = 16; tx <= 32; tx *= 2) {
         const double per_plane = adds + (double)R * (tx + 2 * R) / tx;
         const long long xy = (long long)((g.nx + tx - 1) / tx) * ((g.ny + 128 / tx - 1) / (128 / tx));
-        for (int cz = 1;; cz = cz < 4 ? cz + 1 : cz + cz / 3) {
-            if (cz > g.nz) cz = g.nz;
+        for (int gz = 1; gz <= g.nz && gz <= 1024; ++gz) {
+            const int cz = (g.nz + gz - 1) / gz;
             const long long ctas = xy * ((g.nz + cz - 1) / cz);
             const double dp = 64.0 * ((cz + 2 * R) * per_plane + cz * (fmas + 3.0));
             const double t = (double)((ctas + nsm - 1) / nsm) * dp + 600.0 * (cz + 2 * R);
@@ -278,7 +287,6 @@ void filter_plan(const Geom& g, double r, int nsm, FilterPlan* p) {
                 p->tx = tx;
                 p->cz = cz;
             }
-            if (cz >= g.nz || cz >= 256) break;
         }
     }
 }
