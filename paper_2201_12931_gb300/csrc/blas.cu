@@ -247,17 +247,18 @@ constexpr int kStrip = 4;
 // A = U D U^T (U unit lower) with U^-1 carried along, so that a pivot step is
 // a reciprocal, one rank-one update and one barrier.  16 warps, lane = row:
 // warps 0-7 hold columns w, w + 8, w + 16, w + 24 of A in registers, warps
-// 8-15 those of U^-1.  The chain of 32 pivots bounds it, in latency of FP64
-// instructions (their pipe takes 16 clocks per warp instruction and SM): the
-// columns are published unscaled with 1 / d beside them, and the square
-// roots of the pivots come at the end, all 32 at once: L = U D^(1/2),
-// L^-1 = D^(-1/2) U^-1.  L goes back to the block (zeros above the diagonal),
-// L^-1 to Dk (block kb: TB x TB row-major at Dk + kb TB^2).  A non-positive
-// or non-finite pivot sets info to its row + 1 (first one wins) and continues
+// 8-15 those of U^-1.  The chain of 32 pivots bounds it: FP64 instructions of
+// one warp follow one another in 64 clocks or more.  So the warp of the next
+// pivot updates that column first and publishes it (as it is, and divided by
+// the pivot: U's column) before its other columns, and the square roots of
+// the pivots come at the end, all 32 at once: L = U D^(1/2), L^-1 = D^(-1/2)
+// U^-1.  L goes back to the block (zeros above the diagonal), L^-1 to Dk
+// (block kb: TB x TB row-major at Dk + kb TB^2).  A non-positive or
+// non-finite pivot sets info to its row + 1 (first one wins) and continues
 // with pivot 1.
 __global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int npad, int kb, int* info,
                                                     double* __restrict__ Dk) {
-    __shared__ double col[2][TB], rec[2], piv[TB], root[TB];
+    __shared__ double col[2][TB], ucol[2][TB], piv[TB], root[TB];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, wc = w & 7;
     const bool isA = w < 8;
     const long long base = (long long)kb * TB;
@@ -267,39 +268,41 @@ __global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int 
         const int c = wc + 8 * s;
         a[s] = isA ? A[(base + lane) * npad + base + c] : (lane == c ? 1.0 : 0.0);
     }
+    auto publish = [&](int j, double v) {
+        double d = __shfl_sync(0xffffffffu, v, j);
+        if (!(d > 0.0) || !isfinite(d)) {
+            if (lane == 0) atomicCAS(info, 0, (int)(base + j) + 1);
+            d = 1.0;
+        }
+        const double y = seed_range(d) ? recip_seeded(d) : 1.0 / d;
+        col[j & 1][lane] = v;
+        ucol[j & 1][lane] = v * y;
+        if (lane == 0) piv[j] = d;
+    };
+    if (w == 0) publish(0, a[0]);
 #pragma unroll
-    for (int js = 0; js < 4; ++js)
-        for (int jw = 0; jw < 8; ++jw) {
-            const int j = 8 * js + jw, b = j & 1;
-            if (isA && wc == jw) {
-                double d = __shfl_sync(0xffffffffu, a[js], j);
-                if (!(d > 0.0) || !isfinite(d)) {
-                    if (lane == 0) atomicCAS(info, 0, (int)(base + j) + 1);
-                    d = 1.0;
-                }
-                const double y = seed_range(d) ? recip_seeded(d) : 1.0 / d;
-                col[b][lane] = a[js];
-                if (lane == 0) {
-                    rec[b] = y;
-                    piv[j] = d;
-                }
-            }
-            __syncthreads();
-            const double l = lane > j ? col[b][lane] * rec[b] : 0.0;   // U_ij
+    for (int j = 0; j < TB; ++j) {
+        __syncthreads();
+        const int b = j & 1;
+        const double l = lane > j ? ucol[b][lane] : 0.0;   // U_ij
+        const bool ahead = isA && j + 1 < TB && wc == ((j + 1) & 7);
+        constexpr int kNone = TB;
+        const int next = j + 1 < TB ? (j + 1) >> 3 : 0;
+        if (ahead) {
+            a[next] = fma(-l, col[b][j + 1], a[next]);
+            publish(j + 1, a[next]);
+        }
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const int c = wc + 8 * s;
-                // (c <= j: A's column is done; c > j: U^-1 has a zero in row j)
-                if (isA ? c > j : c <= j) {
-                    const double r = isA ? col[b][c] : __shfl_sync(0xffffffffu, a[s], j);
-                    a[s] = fma(-l, r, a[s]);
-                }
+        for (int s = 0; s < 4; ++s) {
+            const int c = wc + 8 * s;
+            // (c <= j: A's column is done; c > j: U^-1 has a zero in row j)
+            if (isA ? c > (ahead && s == next ? kNone : j) : c <= j) {
+                const double r = isA ? col[b][c] : __shfl_sync(0xffffffffu, a[s], j);
+                a[s] = fma(-l, r, a[s]);
             }
         }
-    if (w == 0) {
-        const double d = piv[lane];   // written by warps that have passed the last barrier
-        root[lane] = rsqrt(d);
     }
+    if (w == 0) root[lane] = rsqrt(piv[lane]);   // (piv written before the last barrier)
     __syncthreads();
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -404,7 +407,8 @@ __global__ void k_transpose(const double* __restrict__ W, double* __restrict__ W
     WT[((long long)bx * TB + ty) * npad + (long long)by * TB + tx] = s[tx][ty];
 }
 
-// y_i = sum_{j<=i} W_ij r_j (lower) or sum_{j>=i} (upper); warp per row.  FP64
+// y_i = sum_{j<=i} W_ij r_order(j) (lower) or u_order(i) = sum_{j>=i} W^T_ij y_j
+// (upper); warp per row.  FP64
 // matrices: FP64 sums.  FP32 matrices: every product and sum with its exact
 // rounding error carried in a second FP32 word (TwoProduct by fused
 // multiply-add, Knuth's TwoSum; the sum is as if accumulated in 48 bits
@@ -417,12 +421,15 @@ __device__ __forceinline__ void two_sum_into(float& s, float& c, float p) {
     s = t;
 }
 template <typename T, bool LOWER>
-__global__ void k_trigemv(int n, int npad, const T* __restrict__ M, const T* __restrict__ v, T* __restrict__ y) {
+__global__ void k_trigemv(int n, int npad, const T* __restrict__ M, const T* __restrict__ v, T* __restrict__ y,
+                          const int* __restrict__ order) {
     const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= n) return;
     const int j0 = LOWER ? 0 : row, j1 = LOWER ? row + 1 : n;
     const T* mr = M + (long long)row * npad;
+    auto at = [&](int j) { return v[LOWER ? order[j] : j]; };
+    T* const dst = y + (LOWER ? row : order[row]);
     if constexpr (std::is_same<T, float>::value) {
         float s[2] = {0.0f, 0.0f}, c[2] = {0.0f, 0.0f};   // two chains
         auto add = [&](int q, float a, float b) {
@@ -436,12 +443,12 @@ __global__ void k_trigemv(int n, int npad, const T* __restrict__ M, const T* __r
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 a[q] = mr[j + 32 * q];
-                b[q] = v[j + 32 * q];
+                b[q] = at(j + 32 * q);
             }
 #pragma unroll
             for (int q = 0; q < 8; ++q) add(q & 1, a[q], b[q]);
         }
-        for (; j < j1; j += 32) add(0, mr[j], v[j]);
+        for (; j < j1; j += 32) add(0, mr[j], at(j));
         c[0] += c[1];
         two_sum_into(s[0], c[0], s[1]);
         for (int o = 16; o > 0; o >>= 1) {
@@ -449,7 +456,7 @@ __global__ void k_trigemv(int n, int npad, const T* __restrict__ M, const T* __r
             c[0] += co;
             two_sum_into(s[0], c[0], so);
         }
-        if (lane == 0) y[row] = s[0] + c[0];
+        if (lane == 0) *dst = s[0] + c[0];
     } else {
         double s[2] = {0.0, 0.0};
         int j = j0 + lane;
@@ -458,14 +465,14 @@ __global__ void k_trigemv(int n, int npad, const T* __restrict__ M, const T* __r
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 a[q] = mr[j + 32 * q];
-                b[q] = v[j + 32 * q];
+                b[q] = at(j + 32 * q);
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) s[q & 1] = fma(a[q], b[q], s[q & 1]);
         }
-        for (; j < j1; j += 32) s[0] = fma(mr[j], v[j], s[0]);
+        for (; j < j1; j += 32) s[0] = fma(mr[j], at(j), s[0]);
         const double t = warp_sum(s[0] + s[1]);
-        if (lane == 0) y[row] = t;
+        if (lane == 0) *dst = t;
     }
 }
 
@@ -610,15 +617,16 @@ void transpose_dense(const Ctx& c, const double* W, double* WT, int npad) {
 }
 
 template <typename T>
-void coarse_apply(const Ctx& c, int n, int npad, const T* W, const T* WT, const T* rhs, T* y, T* out) {
+void coarse_apply(const Ctx& c, const Coarse& cs, const T* W, const T* WT, const T* rhs, T* y, T* out) {
+    const int n = cs.n, npad = cs.npad;
     const unsigned blocks = (unsigned)((n + 3) / 4);   // four rows a block: small grids on all SMs
-    k_trigemv<T, true><<<blocks, 128, 0, c.s>>>(n, npad, W, rhs, y);
+    k_trigemv<T, true><<<blocks, 128, 0, c.s>>>(n, npad, W, rhs, y, cs.order);
     TOPO_LAUNCH_CHECK(c);
-    k_trigemv<T, false><<<blocks, 128, 0, c.s>>>(n, npad, WT, y, out);
+    k_trigemv<T, false><<<blocks, 128, 0, c.s>>>(n, npad, WT, y, out, cs.order);
     TOPO_LAUNCH_CHECK(c);
 }
-template void coarse_apply<double>(const Ctx&, int, int, const double*, const double*, const double*, double*,
+template void coarse_apply<double>(const Ctx&, const Coarse&, const double*, const double*, const double*, double*,
                                    double*);
-template void coarse_apply<float>(const Ctx&, int, int, const float*, const float*, const float*, float*, float*);
+template void coarse_apply<float>(const Ctx&, const Coarse&, const float*, const float*, const float*, float*, float*);
 
 }  // namespace topo

@@ -168,7 +168,7 @@ void free_all(topo_grid* h) {
         F(l.ha); F(l.hb); F(l.Ke64); F(l.Ke32);
     }
     F(h->cs.A); F(h->cs.W64); F(h->cs.WT64); F(h->cs.W32); F(h->cs.WT32); F(h->cs.y64); F(h->cs.y32);
-    F(h->cs.info); F(h->cs.Dk);
+    F(h->cs.info); F(h->cs.order); F(h->cs.Dk);
     F(h->x); F(h->f); F(h->r); F(h->z); F(h->p); F(h->q);
     F(h->r32); F(h->z32); F(h->p32); F(h->q32); F(h->d32); F(h->alpha_hist); F(h->ticket); F(h->el64);
     for (auto& d : h->dring64) F(d);
@@ -216,12 +216,10 @@ topo_status ensure_coarse(topo_grid* h) {
         ALLOC(h, cs.y64, cs.npad);
         ALLOC(h, cs.y32, cs.npad);
         ALLOC(h, cs.info, 1);
+        ALLOC(h, cs.order, cs.npad);
         ALLOC(h, cs.Dk, (size_t)cs.npad * 32);
     }
-    // half-bandwidth of the coarsest matrix: DOFs of nodes up to one step
-    // apart in each direction (node order x fastest, 3 DOFs per node)
-    const int NXc = lc.g.nx + 1, NYc = lc.g.ny + 1;
-    const int band = 3 * (1 + NXc + NXc * NYc) + 2;
+    const int band = coarse_band(lc.g);
     // assembly, Cholesky, L^-1, its transpose and FP32 copies: a fixed
     // sequence of a few hundred small launches, captured once per handle into
     // a CUDA graph and replayed for each new density (the pointers do not
@@ -229,7 +227,7 @@ topo_status ensure_coarse(topo_grid* h) {
     auto body = [&]() {
         const Ctx cc = h->ctx();
         assemble_coarse(cc, lc.g, h->K0d, lc.E64, h->prm.homogenize == 2 && h->L > 1 ? lc.Ke64 : nullptr, lc.mask,
-                        cs.A, cs.npad);
+                        cs.A, cs.npad, cs.order);
         chol_factor(cc, cs.A, cs.npad, band, cs.info, cs.Dk);
         tri_inverse(cc, cs.A, cs.W64, cs.npad, band, cs.Dk);
         transpose_dense(cc, cs.W64, cs.WT64, cs.npad);

@@ -90,6 +90,7 @@ struct Coarse {           // dense coarsest-grid solve: K_c^-1 = W^T W, W = L^-1
     double* y64 = nullptr;    // temporaries of length npad
     float* y32 = nullptr;
     int* info = nullptr;      // device: first non-positive pivot + 1 (0 = ok)
+    int* order = nullptr;     // DOF of the level's node order at each row: nodes run along the shortest axis first
     double* Dk = nullptr;     // inverses of the 32 x 32 diagonal blocks of L (npad x 32)
 };
 
@@ -260,9 +261,14 @@ void tc_b_image(const double* K0, uint32_t* img);
 int stencil_tc(const Ctx& c, int mode, const OpLaunch& L, float kdiag, const float* E, const uint8_t* mask,
                const float* u, const float* f, float* out, float omega, const uint32_t* Bimg, double* dot_partials,
                int* err);
-// dense coarsest operator from E_e K0, or from stored element matrices Ke (non-null)
+// dense coarsest operator from E_e K0, or from stored element matrices Ke (non-null);
+// order (3 * nodes) receives the DOF of each row
 void assemble_coarse(const Ctx& c, const Geom& g, const double* K0, const double* E, const double* Ke,
-                     const uint8_t* mask, double* A, int npad);
+                     const uint8_t* mask, double* A, int npad, int* order);
+// Half-bandwidth of that operator: rows follow the node order with the
+// shortest axis running fastest and the longest slowest, which makes it
+// 3 (1 + N0 + N0 N1) + 2 for the two smaller node counts N0 <= N1
+int coarse_band(const Geom& g);
 // ---- galerkin.cu: stored Galerkin coarse element matrices ------------------
 void galerkin_init_constants();
 // host: the 8 child matrices G_o = P_o^T K0 P_o (8 x 576, o-major)
@@ -342,7 +348,7 @@ void chol_factor(const Ctx& c, double* A, int npad, int band, int* info, double*
 void tri_inverse(const Ctx& c, const double* L, double* W, int npad, int band, const double* Dk);
 void transpose_dense(const Ctx& c, const double* W, double* WT, int npad);
 template <typename T>
-void coarse_apply(const Ctx& c, int n, int npad, const T* W, const T* WT, const T* rhs, T* y, T* out);
+void coarse_apply(const Ctx& c, const Coarse& cs, const T* W, const T* WT, const T* rhs, T* y, T* out);
 
 // message returned by topo_last_error(NULL)
 void set_global_error(const std::string& msg);

@@ -122,7 +122,7 @@ int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot, const D
     const Ctx c = h->ctx();
     Level& lv = h->lev[l];
     if (l == h->L - 1) {
-        coarse_apply<T>(c, h->cs.n, h->cs.npad, P<T>::W(h), P<T>::WT(h), f, P<T>::y(h), out);
+        coarse_apply<T>(c, h->cs, P<T>::W(h), P<T>::WT(h), f, P<T>::y(h), out);
         if (dot) dot_partials<T, T>(c, 3 * lv.g.nn, f, out, dot);
         return dot ? kRedBlocks : 0;
     }
@@ -224,7 +224,7 @@ static bf16* vcycle_lp(topo_grid* h, int l, const float* f, float* out_f, double
     }
     restrict_residual<float>(c, lv.g, lv.mask, lc.mask, res, lc.v32.f);
     if (l + 1 == h->L - 1) {
-        coarse_apply<float>(c, h->cs.n, h->cs.npad, h->cs.W32, h->cs.WT32, lc.v32.f, h->cs.y32, lc.v32.a);
+        coarse_apply<float>(c, h->cs, h->cs.W32, h->cs.WT32, lc.v32.f, h->cs.y32, lc.v32.a);
         prolong_add_bf16<float>(c, lv.g, lv.mask, lc.mask, lc.v32.a, cur);
     } else {
         int npc = 0;
@@ -255,7 +255,7 @@ int vcycle_bf16(topo_grid* h, int l, const float* f, float* out, double* dot) {
     const Ctx c = h->ctx();
     Level& lv = h->lev[l];
     if (l == h->L - 1) {   // single level: the direct solve
-        coarse_apply<float>(c, h->cs.n, h->cs.npad, h->cs.W32, h->cs.WT32, f, h->cs.y32, out);
+        coarse_apply<float>(c, h->cs, h->cs.W32, h->cs.WT32, f, h->cs.y32, out);
         if (dot) dot_partials<float, float>(c, 3 * lv.g.nn, f, out, dot);
         return dot ? kRedBlocks : 0;
     }

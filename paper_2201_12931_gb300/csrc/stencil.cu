@@ -6,6 +6,7 @@
 //
 // Operator with Dirichlet rows: y = P_f K P_f u + (I - P_f) u, P_f zeroing the
 // fixed DOFs, K = sum_e E_e A_e^T K0 A_e (E_e already holds 2^l on level l).
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -453,9 +454,15 @@ void launch_mode(const Ctx& c, const OpLaunch& L, const ModalK<T>& mk, const T* 
 // node, column component) gathers, in a fixed order, the <= 8 elements that
 // contain both nodes -- element matrices E_e K0, or the stored Ke[e] of a
 // Galerkin level.  Rows and columns of fixed DOFs stay zero here.
+// row of a node's first DOF / 3: nodes numbered along the shortest axis first
+struct NodeOrder {
+    int sx, sy, sz;
+    __device__ int at(int i, int j, int k) const { return sx * i + sy * j + sz * k; }
+};
+
 __global__ void k_assemble(const double* __restrict__ K0, const double* __restrict__ E,
                            const double* __restrict__ Ke, const uint8_t* __restrict__ mask, double* __restrict__ A,
-                           int nx, int ny, int nz, int npad) {
+                           int nx, int ny, int nz, int npad, NodeOrder no) {
     const int NX = nx + 1, NY = ny + 1, NZ = nz + 1;
     const long long total = 3LL * NX * NY * NZ * 81;
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -482,13 +489,22 @@ __global__ void k_assemble(const double* __restrict__ K0, const double* __restri
                 const int r = 3 * a + c, s = 3 * b + d;
                 v += Ke ? Ke[e * 576 + r * 24 + s] : E[e] * K0[r * 24 + s];
             }
-    A[(3 * nr + c) * (long long)npad + 3 * nc + d] = v;
+    A[(3 * no.at(i, j, k) + c) * (long long)npad + 3 * no.at(i2, j2, k2) + d] = v;
 }
 
-__global__ void k_assemble_diag(const uint8_t* __restrict__ mask, double* __restrict__ A, int n, int npad) {
+// unit diagonal of fixed and padding rows, and the DOF of every row
+__global__ void k_assemble_diag(const uint8_t* __restrict__ mask, double* __restrict__ A, int nx, int ny, int nz, int npad,
+                                NodeOrder no, int* __restrict__ order) {
     const int d = blockIdx.x * blockDim.x + threadIdx.x;
     if (d >= npad) return;
-    if (d >= n || ((mask[d / 3] >> (d % 3)) & 1u)) A[(long long)d * npad + d] = 1.0;
+    const int NX = nx + 1, NY = ny + 1, n = 3 * NX * NY * (nz + 1);
+    int row = d;
+    if (d < n) {
+        const int node = d / 3;
+        row = 3 * no.at(node % NX, node / NX % NY, node / (NX * NY)) + d % 3;
+        order[row] = d;
+    }
+    if (d >= n || ((mask[d / 3] >> (d % 3)) & 1u)) A[(long long)row * npad + row] = 1.0;
 }
 
 // rho^p by repeated multiplication for integer p (FP64 pow is slow on GB300)
@@ -705,13 +721,33 @@ int stencil_df(const Ctx& c, int mode, const OpLaunch& L, const ModalK<dfl>& mk,
     return dot ? L.gx * L.gy * L.gz : 0;
 }
 
+// strides of the three axes in the row order, and the two smaller node counts
+static NodeOrder node_order(const Geom& g, int* small) {
+    const int N[3] = {g.NX(), g.NY(), g.NZ()};
+    int ax[3] = {0, 1, 2}, stride[3];
+    std::stable_sort(ax, ax + 3, [&](int a, int b) { return N[a] < N[b]; });
+    for (int q = 0, s = 1; q < 3; s *= N[ax[q++]]) stride[ax[q]] = s;
+    if (small) {
+        small[0] = N[ax[0]];
+        small[1] = N[ax[1]];
+    }
+    return NodeOrder{stride[0], stride[1], stride[2]};
+}
+
+int coarse_band(const Geom& g) {
+    int n[2];
+    node_order(g, n);
+    return 3 * (1 + n[0] + n[0] * n[1]) + 2;
+}
+
 void assemble_coarse(const Ctx& c, const Geom& g, const double* K0, const double* E, const double* Ke,
-                     const uint8_t* mask, double* A, int npad) {
+                     const uint8_t* mask, double* A, int npad, int* order) {
+    const NodeOrder no = node_order(g, nullptr);
     cudaMemsetAsync(A, 0, sizeof(double) * (size_t)npad * npad, c.s);
     const long long total = 3 * g.nn * 81;
-    k_assemble<<<(unsigned)((total + 255) / 256), 256, 0, c.s>>>(K0, E, Ke, mask, A, g.nx, g.ny, g.nz, npad);
+    k_assemble<<<(unsigned)((total + 255) / 256), 256, 0, c.s>>>(K0, E, Ke, mask, A, g.nx, g.ny, g.nz, npad, no);
     TOPO_LAUNCH_CHECK(c);
-    k_assemble_diag<<<(npad + 255) / 256, 256, 0, c.s>>>(mask, A, (int)(3 * g.nn), npad);
+    k_assemble_diag<<<(npad + 255) / 256, 256, 0, c.s>>>(mask, A, g.nx, g.ny, g.nz, npad, no, order);
     TOPO_LAUNCH_CHECK(c);
 }
 
