@@ -34,7 +34,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 
 // Element-column z-march operator kernel; see operator.cuh for the scheme.
 // The per-plane body is a generic lambda called with a compile-time buffer
-// parity B = P & 1, so that double buffers and the two-plane register history
+// parity B, so that double buffers and the two-plane register history
 // are addressed statically (no register moves, no dynamic indexing).
 // T: arithmetic, f, E; TU: storage of u; TO: storage of the output.
 template <typename T, typename TU, typename TO, int MODE, bool DOT>
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     T stE = T(0);
     double dot = 0.0;
     [[maybe_unused]] float dotf = 0.0f;
-    // per-plane register slots, slot = plane & 3: own node raw u, f, mask,
+    // per-plane register slots, slot = (plane - first) & 3: own node raw u, f, mask,
     // the column modulus of the layer below the plane, and (two slots) the
     // halo node; planes P-2 .. P+1 are live in step P, so no copies occur.
     // Double-FP32 arithmetic keeps the loaded FP64 words in the slots and
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
         sE[S] = (col_ok && P >= 1 && P <= nz) ? (TSl)E[(Ix)(P - 1) * nx * ny + col_xy] : TSl(0);
     };
 
-    // step of node plane P, B = P & 3 (static)
+    // step of node plane P, B = (P - first plane) & 3 (static)
     auto step = [&](auto Bc, int P) {
         constexpr int B = decltype(Bc)::value;
         constexpr int B2 = B & 1;                 // shared-memory buffer
@@ -390,17 +390,12 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     using S1 = std::integral_constant<int, 1>;
     using S2 = std::integral_constant<int, 2>;
     using S3 = std::integral_constant<int, 3>;
-    // planes kz0-1 .. kz1+1 are processed; the range is widened to whole
-    // groups of four (P = 0 mod 4 first) -- the extra steps are guarded no-ops
+    // planes kz0-1 .. kz1+1 in groups of four, the slots counted from the first
+    // one (the steps past the last are guarded no-ops; op_launch favours chunks
+    // without them)
     const int Pfirst = kz0 - 1;
-    int P = Pfirst - (((Pfirst % 4) + 4) % 4);
-    switch (Pfirst - P) {   // prefetch plane Pfirst into its slot
-        case 0: fetch(S0{}, Pfirst); break;
-        case 1: fetch(S1{}, Pfirst); break;
-        case 2: fetch(S2{}, Pfirst); break;
-        default: fetch(S3{}, Pfirst); break;
-    }
-    for (; P <= kz1 + 1; P += 4) {
+    fetch(S0{}, Pfirst);
+    for (int P = Pfirst; P <= kz1 + 1; P += 4) {
         step(S0{}, P);
         step(S1{}, P + 1);
         step(S2{}, P + 2);
@@ -623,10 +618,13 @@ __global__ void __launch_bounds__(256) k_energy_sens_z(ModalCoef mc, const doubl
 }  // namespace
 
 // Launch geometry: x-y tiles of (kOpTX - 1) x (ty - 1) output node columns
-// and z chunks of at least 16 planes (each chunk recomputes one layer and
-// pays about 4.5 extra exchange steps).  At least target_ctas CTAs; beyond
-// that the number of chunks minimises (waves of resident CTAs) x (steps per
-// CTA), so that a last, nearly empty wave does not cost a whole CTA time.
+// and z chunks.  A chunk of cz planes marches over cz + 3 of them, in groups
+// of four (kernels count the groups from the chunk's first plane).  At least
+// target_ctas CTAs where the grid allows; beyond that the number of chunks
+// minimises (waves of resident CTAs) x (steps per CTA), so that neither a
+// nearly empty last wave nor a nearly empty last group costs a whole one:
+// 128x64x64 elements take chunks of 5 planes (8 steps) instead of 4 (12
+// steps while groups began at multiples of four).
 OpLaunch op_launch(const Geom& g, int ty, int target_ctas, int resident_ctas) {
     OpLaunch L;
     L.g = g;
@@ -649,7 +647,7 @@ OpLaunch op_launch(const Geom& g, int ty, int target_ctas, int resident_ctas) {
         const int cz = chunk(gz);
         const long long gz_eff = (NZ + cz - 1) / cz;
         const long long waves = (xy * gz_eff + resident_ctas - 1) / resident_ctas;
-        const double cost = (double)waves * (cz + 4.5);
+        const double cost = (double)waves * ((cz + 6) / 4 * 4 + 1.5);
         if (best_cost < 0.0 || cost < best_cost) {
             best_cost = cost;
             best_cz = cz;
