@@ -86,8 +86,10 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     // which it needs fewer registers (measured: 32-bit spilled and was slower)
     using Ix = std::conditional_t<PUPD, long long, int>;
     const Ix nplane = (Ix)NX * NY;
-    const int own_xy = node_ok ? in + NX * jn : 0;
-    const int halo_xy = halo_ok ? hx + NX * hy : 0;
+    // nodes outside the grid read the nearest one inside (their elements have
+    // modulus 0): no predicates and zero fills around the loads
+    const int own_xy = min(max(in, 0), NX - 1) + NX * min(max(jn, 0), NY - 1);
+    const int halo_xy = min(max(hx, 0), NX - 1) + NX * min(max(hy, 0), NY - 1);
     const int col_xy = col_ok ? in + nx * jn : 0;
     const int uoff = (ty * (TX + 1) + tx) * 4;      // own slot in a plane buffer
     const int hoff = (hsy * (TX + 1) + hsx) * 4;    // halo slot
@@ -135,53 +137,48 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     // load plane P into slot S (plane-uniform base + per-thread offset)
     auto fetch = [&](auto Sc, int P) {
         constexpr int S = decltype(Sc)::value;
-        const bool pin = P >= 0 && P <= nz;
-        const Ix pb = (Ix)P * nplane;
+        const Ix pb = (Ix)min(max(P, 0), nz) * nplane;   // (as for nodes: the nearest plane)
         if constexpr (kDF) {
             // raw FP64 words: own and halo node, the plane's reference (tile
             // corner node); f is loaded by the step (one plane behind)
-            const bool ok = pin && node_ok;
-            sm[S] = ok ? mask[pb + own_xy] : 0u;
+            sm[S] = mask[pb + own_xy];
             const TU* ub = u + 3 * pb + own3;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                su[S][c] = ok ? (double)ub[c] : 0.0;
-                srf[S & 1][c] = pin ? (double)u[3 * pb + ref3 + c] : 0.0;
+                su[S][c] = (double)ub[c];
+                srf[S & 1][c] = (double)u[3 * pb + ref3 + c];
             }
-            const bool okh = pin && halo_ok;
-            shm[S & 1] = okh ? mask[pb + halo_xy] : 0u;
-            const TU* hb = u + 3 * pb + halo3;
+            if (halo_warp) {
+                shm[S & 1] = mask[pb + halo_xy];
+                const TU* hb = u + 3 * pb + halo3;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) shv[S & 1][c] = okh ? (double)hb[c] : 0.0;
+                for (int c = 0; c < 3; ++c) shv[S & 1][c] = (double)hb[c];
+            }
         } else if (NEEDU || NEEDF) {
-            const bool ok = pin && node_ok;
-            sm[S] = ok ? mask[pb + own_xy] : 0u;
+            sm[S] = mask[pb + own_xy];
             const TU* ub = u + 3 * pb + own3;
             const typename OpStore<T>::type* fb_ = f + 3 * pb + own3;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                if (NEEDU && !J2) su[S][c] = ok ? (T)ldv(ub + c) : T(0);
-                if (NEEDF) sf[S][c] = ok ? (T)fb_[c] : T(0);
+                if (NEEDU && !J2) su[S][c] = (T)ldv(ub + c);
+                if (NEEDF) sf[S][c] = (T)fb_[c];
             }
-            if constexpr (J2) sdv[S] = ok ? (T)Dinv[pb + own_xy] : T(0);
+            if constexpr (J2) sdv[S] = (T)Dinv[pb + own_xy];
         }
-        // residual and K.u: the halo loads behind a warp-uniform branch (two of
-        // the eight warps hold halo threads); measured faster there, slower in
-        // the Jacobi and fused modes
-        [[maybe_unused]] constexpr bool kHaloBranch = (MODE == ST_RESID || MODE == ST_APPLY);
-        if constexpr (NEEDU && !kDF) if (!kHaloBranch || halo_warp) {
-            const bool okh = pin && halo_ok;
-            shm[S & 1] = okh ? mask[pb + halo_xy] : 0u;
+        // halo loads behind a warp-uniform branch (two of the eight warps hold
+        // halo threads; the others would load real nodes here)
+        if constexpr (NEEDU && !kDF) if (halo_warp) {
+            shm[S & 1] = mask[pb + halo_xy];
             [[maybe_unused]] const TU* hb = u + 3 * pb + halo3;
             if constexpr (!J2) {
 #pragma unroll
-                for (int c = 0; c < 3; ++c) shv[S & 1][c] = okh ? (T)ldv(hb + c) : T(0);
+                for (int c = 0; c < 3; ++c) shv[S & 1][c] = (T)ldv(hb + c);
             }
             if constexpr (PUPD || J2) {
                 const typename OpStore<T>::type* hf = f + 3 * pb + halo3;
 #pragma unroll
-                for (int c = 0; c < 3; ++c) shf[S & 1][c] = okh ? (T)hf[c] : T(0);
-                if constexpr (J2) shd[S & 1] = okh ? (T)Dinv[pb + halo_xy] : T(0);
+                for (int c = 0; c < 3; ++c) shf[S & 1][c] = (T)hf[c];
+                if constexpr (J2) shd[S & 1] = (T)Dinv[pb + halo_xy];
             }
         }
         sE[S] = (col_ok && P >= 1 && P <= nz) ? (TSl)E[(Ix)(P - 1) * nx * ny + col_xy] : TSl(0);
@@ -296,32 +293,37 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
             TO* o = out + 3 * ((Ix)Q * nplane) + own3;
             const unsigned m2 = sm[SO];
             typename DotAcc<T>::type d32 = 0;
+            T r[3];
+            [[maybe_unused]] T uo[3], fo[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const bool fixed = (m2 >> c) & 1u;
-                [[maybe_unused]] T uo;
-                [[maybe_unused]] const T fo = T(sf[SO][c]);
-                if constexpr (kDF) {   // fixed rows read u itself (the slots are not kept)
-                    uo = fixed ? T((double)u[3 * ((Ix)Q * nplane) + own3 + c]) : T(0);
-                } else {
-                    uo = su[SO][c];
+                fo[c] = T(sf[SO][c]);
+                if constexpr (!kDF) uo[c] = su[SO][c];
+                if constexpr (MODE == ST_APPLY || MODE == ST_APPLY_P) r[c] = y[c];
+                else if constexpr (MODE == ST_RESID) r[c] = fo[c] - y[c];
+                else if constexpr (MODE == ST_JACOBI || MODE == ST_JACOBI2) r[c] = uo[c] + omega * (fo[c] - y[c]) * rD;
+                else r[c] = omega * fo[c] * rD;
+            }
+            if (m2) {   // identity rows of fixed DOFs, off the common path
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    if ((m2 >> c) & 1u) {
+                        if constexpr (kDF) uo[c] = T((double)u[3 * ((Ix)Q * nplane) + own3 + c]);   // (not kept in slots)
+                        if constexpr (MODE == ST_APPLY || MODE == ST_APPLY_P) r[c] = uo[c];
+                        else if constexpr (MODE == ST_RESID) r[c] = fo[c] - uo[c];
+                        else if constexpr (MODE == ST_JACOBI || MODE == ST_JACOBI2) r[c] = uo[c] + omega * (fo[c] - uo[c]);
+                        else r[c] = omega * fo[c];
+                    }
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if constexpr (DOT) {
+                    if constexpr (MODE == ST_APPLY || MODE == ST_APPLY_P) d32 += to_acc(uo[c]) * to_acc(r[c]);
+                    else if constexpr (MODE == ST_RESID) d32 += to_acc(r[c]) * to_acc(r[c]);
+                    else d32 += fo[c] * r[c];
                 }
-                T r;
-                if constexpr (MODE == ST_APPLY || MODE == ST_APPLY_P) {
-                    r = fixed ? uo : y[c];
-                    if (DOT) d32 += to_acc(uo) * to_acc(r);
-                    if constexpr (PUPD) stv(pout + 3 * ((Ix)Q * nplane) + own3 + c, uo);
-                } else if constexpr (MODE == ST_RESID) {
-                    r = fo - (fixed ? uo : y[c]);
-                    if (DOT) d32 += to_acc(r) * to_acc(r);
-                } else if constexpr (MODE == ST_JACOBI || MODE == ST_JACOBI2) {
-                    r = fixed ? uo + omega * (fo - uo) : uo + omega * (fo - y[c]) * rD;
-                    if (DOT) d32 += fo * r;
-                } else {
-                    r = omega * fo * (fixed ? T(1) : rD);
-                    if (DOT) d32 += fo * r;
-                }
-                stv(o + c, r);
+                if constexpr (PUPD) stv(pout + 3 * ((Ix)Q * nplane) + own3 + c, uo[c]);
+                stv(o + c, r[c]);
             }
             if constexpr (DOT) {
                 // FP32 kernels: FP32 per thread (one column of a z chunk),
