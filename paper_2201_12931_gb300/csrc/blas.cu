@@ -218,10 +218,26 @@ __global__ void k_update_p(long long n, const Scalars* __restrict__ sc, const T*
         p[i] = z[i] + b * p[i];
 }
 
+// FP64 <-> FP32 conversion instructions run at the FP64 rate, which bounds a
+// pass of 12 bytes per value (12.8M values: 26 us); narrow() and widen() are
+// the same values from integer instructions
 template <typename S, typename D>
-__global__ void k_convert(long long n, const S* __restrict__ s, D* __restrict__ d) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        d[i] = (D)s[i];
+__global__ void __launch_bounds__(256) k_convert(long long n, const S* __restrict__ s, D* __restrict__ d) {
+    auto conv = [](S v) -> D {
+        if constexpr (std::is_same<S, double>::value && std::is_same<D, float>::value) return narrow(v);
+        else if constexpr (std::is_same<S, float>::value && std::is_same<D, double>::value) return widen(v);
+        else return (D)v;
+    };
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (; i + 3 * stride < n; i += 4 * stride) {   // four loads in flight
+        S v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = s[i + q * stride];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) d[i + q * stride] = conv(v[q]);
+    }
+    for (; i < n; i += stride) d[i] = conv(s[i]);
 }
 
 __global__ void k_fill(long long n, double* __restrict__ v, double value) {
@@ -460,15 +476,15 @@ __global__ void k_trigemv(int n, int npad, const T* __restrict__ M, const T* __r
     } else {
         double s[2] = {0.0, 0.0};
         int j = j0 + lane;
-        for (; j + 96 < j1; j += 128) {
-            double a[4], b[4];
+        for (; j + 224 < j1; j += 256) {
+            double a[8], b[8];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = 0; q < 8; ++q) {
                 a[q] = mr[j + 32 * q];
                 b[q] = at(j + 32 * q);
             }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) s[q & 1] = fma(a[q], b[q], s[q & 1]);
+            for (int q = 0; q < 8; ++q) s[q & 1] = fma(a[q], b[q], s[q & 1]);
         }
         for (; j < j1; j += 32) s[0] = fma(mr[j], at(j), s[0]);
         const double t = warp_sum(s[0] + s[1]);
@@ -545,7 +561,8 @@ template void cg_flush_x<float>(const Ctx&, long long, float* const*, const doub
 
 template <typename S, typename D>
 void convert(const Ctx& c, long long n, const S* src, D* dst) {
-    k_convert<S, D><<<grid_for(n, 256) > 8192 ? 8192 : grid_for(n, 256), 256, 0, c.s>>>(n, src, dst);
+    const unsigned g = grid_for(n, 1024);
+    k_convert<S, D><<<g > kUpdateBlocks ? kUpdateBlocks : g, 256, 0, c.s>>>(n, src, dst);
     TOPO_LAUNCH_CHECK(c);
 }
 template void convert<double, float>(const Ctx&, long long, const double*, float*);

@@ -21,6 +21,24 @@ __device__ __forceinline__ double widen_f32(float v) {
     const unsigned b = __float_as_uint(v);
     return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
 }
+// The conversions (float)v and (double)v bit for bit on integer words; values
+// outside FP32's normal range (other than zeros) take the instructions
+__device__ __forceinline__ float narrow(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    if (((hi >> 20) & 0x7ffu) - 897u < 254u) {
+        unsigned b = (__funnelshift_l(lo, hi & 0x7fffffffu, 3) - 0xc0000000u);   // truncated magnitude
+        b += (lo << 3) + (b & 1u) > 0x80000000u ? 1u : 0u;                       // to nearest, ties to even
+        return __uint_as_float(b | (hi & 0x80000000u));
+    }
+    if (((hi & 0x7fffffffu) | lo) == 0u) return __uint_as_float(hi);
+    return (float)v;
+}
+__device__ __forceinline__ double widen(float v) {
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if ((m >> 23) - 1u < 254u) return __hiloint2double((int)(((m >> 3) + (896u << 20)) | (b & 0x80000000u)), (int)(b << 29));
+    if (m == 0u) return __hiloint2double((int)b, 0);
+    return (double)v;
+}
 // 1 / b by two Newton steps from the FP32 reciprocal, for 2^-100 <= b < 2^100
 __device__ __forceinline__ double recip_seeded(double b) {
     float r;
