@@ -23,8 +23,12 @@ inline unsigned grid_for(long long n, int threads) {
 // a chunk of coarse planes.  s_k = the masked in-plane 3 x 3 sum (weights
 // 1, 1/2) of fine plane k around (2I, 2J); r_c(K) = s_{2K-1}/2 + s_{2K} +
 // s_{2K+1}/2, and s_{2K+1} is reused as the lower plane of K + 1, so every
-// fine plane is summed once per coarse column.
-template <typename T>
+// fine plane is summed once per coarse column.  EARLY: the nine values and
+// masks of a plane are loaded before any is used (a value is not loaded behind
+// its mask): a small level's launch is as long as its chain of loads (33x17x17
+// coarse nodes: 10.9 -> 6.9 us); where the grid fills the GPU the extra
+// registers cost more.
+template <typename T, bool EARLY>
 __global__ void __launch_bounds__(256) k_restrict_z(const uint8_t* __restrict__ maskf, const uint8_t* __restrict__ maskc,
                                                     const T* __restrict__ rf, T* __restrict__ rc, int nxf, int nyf,
                                                     int nzf, int czc) {
@@ -34,29 +38,45 @@ __global__ void __launch_bounds__(256) k_restrict_z(const uint8_t* __restrict__ 
     if (I >= NXc || J >= NYc) return;
     const int K0 = blockIdx.z * czc, K1 = min(K0 + czc, NZc);
     const long long fplane = (long long)NXf * NYf;
-    // the nine values and masks of a plane are loaded before any is used (a
-    // value is not loaded behind its mask): on small levels the launch is as
-    // long as its chain of loads
     auto plane_sum = [&](int k, T* s) {
         s[0] = s[1] = s[2] = T(0);
         if (k < 0 || k > nzf) return;
-        T v[9][3];
-        unsigned m[9];
+        if constexpr (EARLY) {
+            T v[9][3];
+            unsigned m[9];
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const int i = 2 * I + q % 3 - 1, j = 2 * J + q / 3 - 1;
-            const bool ok = i >= 0 && i < NXf && j >= 0 && j < NYf;
-            const long long n = ok ? i + (long long)NXf * j + fplane * k : 0;
-            m[q] = ok ? maskf[n] : 7u;
+            for (int q = 0; q < 9; ++q) {
+                const int i = 2 * I + q % 3 - 1, j = 2 * J + q / 3 - 1;
+                const bool ok = i >= 0 && i < NXf && j >= 0 && j < NYf;
+                const long long n = ok ? i + (long long)NXf * j + fplane * k : 0;
+                m[q] = ok ? maskf[n] : 7u;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) v[q][c] = rf[3 * n + c];
+                for (int c = 0; c < 3; ++c) v[q][c] = rf[3 * n + c];
+            }
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                const T w = (q % 3 != 1 ? T(0.5) : T(1)) * (q / 3 != 1 ? T(0.5) : T(1));
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    if (!((m[q] >> c) & 1u)) s[c] += w * v[q][c];
+            }
+            return;
         }
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const T w = (q % 3 != 1 ? T(0.5) : T(1)) * (q / 3 != 1 ? T(0.5) : T(1));
+        for (int dy = -1; dy <= 1; ++dy) {
+            const int j = 2 * J + dy;
+            if (j < 0 || j >= NYf) continue;
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
-                if (!((m[q] >> c) & 1u)) s[c] += w * v[q][c];
+            for (int dx = -1; dx <= 1; ++dx) {
+                const int i = 2 * I + dx;
+                if (i < 0 || i >= NXf) continue;
+                const T w = (dx ? T(0.5) : T(1)) * (dy ? T(0.5) : T(1));
+                const long long n = i + (long long)NXf * j + fplane * k;
+                const unsigned mf = maskf[n];
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    if (!((mf >> c) & 1u)) s[c] += w * rf[3 * n + c];
+            }
         }
     };
     T lo[3], mid[3], hi[3];
@@ -270,7 +290,8 @@ void restrict_residual(const Ctx& c, const Geom& gf, const uint8_t* maskf, const
                        T* rc) {
     const int czc = transfer_cz((long long)(gf.nx / 2 + 1) * (gf.ny / 2 + 1), gf.nz / 2 + 1, kRestrictCz);
     const dim3 grid((gf.nx / 2 + 1 + 31) / 32, (gf.ny / 2 + 1 + 7) / 8, (gf.nz / 2 + 1 + czc - 1) / czc);
-    k_restrict_z<T><<<grid, dim3(32, 8), 0, c.s>>>(maskf, maskc, rf, rc, gf.nx, gf.ny, gf.nz, czc);
+    if (czc == 1) k_restrict_z<T, true><<<grid, dim3(32, 8), 0, c.s>>>(maskf, maskc, rf, rc, gf.nx, gf.ny, gf.nz, czc);
+    else k_restrict_z<T, false><<<grid, dim3(32, 8), 0, c.s>>>(maskf, maskc, rf, rc, gf.nx, gf.ny, gf.nz, czc);
     TOPO_LAUNCH_CHECK(c);
 }
 template void restrict_residual<double>(const Ctx&, const Geom&, const uint8_t*, const uint8_t*, const double*,
