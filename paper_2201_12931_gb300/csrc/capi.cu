@@ -174,7 +174,7 @@ void free_all(topo_grid* h) {
     for (auto& d : h->dring64) F(d);
     for (auto& d : h->dring32) F(d);
     F(h->K0d); F(h->K0f);
-    F(h->dc_work); F(h->xnew_work); F(h->oc_hi); F(h->G64); F(h->oc_dv); F(h->stab); F(h->dv_cache);
+    F(h->dc_work); F(h->xnew_work); F(h->oc_hi); F(h->G64); F(h->oc_dv); F(h->stab); F(h->dv_cache); F(h->rdv_cache);
     F(h->lam); F(h->oc_ws); F(h->dtmp); F(h->dflag); F(h->tc_err); F(h->tcB); F(h->partials); F(h->sc);
     if (h->host_sc) cudaFreeHost(h->host_sc);
     delete h->mk64;
@@ -263,11 +263,15 @@ topo_status prepare_filter(topo_grid* h, double r) {
     return TOPO_OK;
 }
 
-// H^T 1, the volume sensitivity of the OC update, for the radius prepared last
-void prepare_dv(topo_grid* h) {
-    if (h->dv_radius == h->S_radius) return;
+// H^T 1, the volume sensitivity of the OC update, and its reciprocal for the
+// radius prepared last
+topo_status prepare_dv(topo_grid* h) {
+    if (h->dv_radius == h->S_radius) return TOPO_OK;
+    if (!h->rdv_cache) ALLOC(h, h->rdv_cache, h->lev[0].g.ne);
     filter_launch(h->ctx(), h->lev[0].g, h->filt, 1, nullptr, nullptr, 0.0, h->stab, h->dv_cache);
+    reciprocal(h->ctx(), h->lev[0].g.ne, h->dv_cache, h->rdv_cache);
     h->dv_radius = h->S_radius;
+    return TOPO_OK;
 }
 
 // Operator coefficients of operator.cuh from the modal blocks; checks the
@@ -788,10 +792,11 @@ topo_status topo_oc_update(topo_handle h, double r, double move, double volfrac,
     if (s != TOPO_OK) return s;
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
-    prepare_dv(h);
+    s = prepare_dv(h);
+    if (s != TOPO_OK) return s;
     filter_launch(c, g, h->filt, 1, dc_dev, nullptr, 0.0, h->stab, h->dc_work);
     // q over dc_work, lower bounds in xnew_work, upper bounds in oc_hi
-    oc_prepare(c, g.ne, rho_dev_inout, h->dc_work, h->dc_work, h->dv_cache, nullptr, move, h->xnew_work, h->oc_hi,
+    oc_prepare(c, g.ne, rho_dev_inout, h->dc_work, h->dc_work, h->dv_cache, h->rdv_cache, nullptr, move, h->xnew_work, h->oc_hi,
                h->r, h->oc_ws);
     return oc_bisection(h, volfrac, rho_dev_inout, h->dv_cache, change_out, (double)g.ne);
 }
@@ -808,7 +813,7 @@ topo_status topo_oc_update_unfiltered(topo_handle h, double move, double volfrac
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
     if (passive_dev && !h->oc_dv) ALLOC(h, h->oc_dv, g.ne);
-    oc_prepare(c, g.ne, rho_dev_inout, dc_dev, h->dc_work, passive_dev ? h->oc_dv : nullptr, passive_dev, move,
+    oc_prepare(c, g.ne, rho_dev_inout, dc_dev, h->dc_work, passive_dev ? h->oc_dv : nullptr, nullptr, passive_dev, move,
                h->xnew_work, h->oc_hi, h->r, h->oc_ws);
     if (!passive_dev) return oc_bisection(h, volfrac, rho_dev_inout, nullptr, change_out, (double)g.ne);
     dot_partials<double, double>(c, g.ne, h->oc_dv, h->oc_dv, h->partials);   // number of active elements

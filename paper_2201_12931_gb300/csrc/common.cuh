@@ -158,6 +158,7 @@ struct topo_grid {
     topo::FilterPlan filt{};        // weights and launch geometry of the filter for S_radius
     double* stab = nullptr;         // its table of weight sums (2 kFilterTab)
     double* dv_cache = nullptr;     // H^T 1 for dv_radius
+    double* rdv_cache = nullptr;    // its reciprocal (on first use)
     double S_radius = -1.0, dv_radius = -1.0;
     int nsm = 152;                  // multiprocessors of the device
     double* lam = nullptr;          // OC bisection state (device)
@@ -364,10 +365,11 @@ void filter_launch(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, c
 // ---- oc.cu ---------------------------------------------------------------
 // OC update: q = x sqrt(max(-dc~, 1e-30) / dv~) (in place over dc~ allowed),
 // move-limit bounds lo / hi, and FP32 copies of (q, lo, hi, dv) in pack (16 B
-// per element).  dv null: 1 (the volume of x itself); passive (0 active, 1
+// per element).  dv null: 1 (the volume of x itself), else rdv = 1 / dv; passive (0 active, 1
 // solid, 2 void): lo = hi = 1 / 0, q = 0, and dv is written (0; active: 1).
 void oc_prepare(const Ctx& c, long long ne, const double* x, const double* dct, double* q, double* dv,
-                const uint8_t* passive, double move, double* lo, double* hi, void* pack, void* search);
+                const double* rdv, const uint8_t* passive, double move, double* lo, double* hi, void* pack, void* search);
+void reciprocal(const Ctx& c, long long n, const double* v, double* r);
 // the multiplier with sum dv clamp(q lambda^(-1/2), lo, hi) = target: screening
 // passes in FP32, then the bisection on [0, 1e9] with exact volumes; result
 // and success in the search state (oc_search_bytes of device memory)
