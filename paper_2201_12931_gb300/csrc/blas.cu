@@ -424,71 +424,78 @@ __global__ void k_transpose(const double* __restrict__ W, double* __restrict__ W
 }
 
 // y_i = sum_{j<=i} W_ij r_order(j) (lower) or u_order(i) = sum_{j>=i} W^T_ij y_j
-// (upper); warp per row.  FP64
-// matrices: FP64 sums.  FP32 matrices: every product and sum with its exact
-// rounding error carried in a second FP32 word (TwoProduct by fused
+// (upper); a block of 128 threads per row.  What bounds it is the latency of a
+// row's loads: with a warp per row, a row of 1911 was a chain of up to 8
+// batches of loads (and of the order behind them: 22 us), now of two.
+// FP64 matrices: FP64 sums.  FP32 matrices: every product and sum with its
+// exact rounding error carried in a second FP32 word (TwoProduct by fused
 // multiply-add, Knuth's TwoSum; the sum is as if accumulated in 48 bits
 // before the one rounding of the result): 9 FP32 instructions per entry
 // where two conversions and an FP64 multiply-add take 48 issue cycles of the
-// SM, which bounded the product (25 us for 1911 rows).
+// SM.
 __device__ __forceinline__ void two_sum_into(float& s, float& c, float p) {
     const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
     c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b)));
     s = t;
 }
+constexpr int kGemv = 128;
 template <typename T, bool LOWER>
-__global__ void k_trigemv(int n, int npad, const T* __restrict__ M, const T* __restrict__ v, T* __restrict__ y,
-                          const int* __restrict__ order) {
-    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (row >= n) return;
-    const int j0 = LOWER ? 0 : row, j1 = LOWER ? row + 1 : n;
+__global__ void __launch_bounds__(kGemv) k_trigemv(int n, int npad, const T* __restrict__ M, const T* __restrict__ v,
+                                                   T* __restrict__ y, const int* __restrict__ order) {
+    __shared__ T red[2][kGemv / 32];
+    const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int j1 = LOWER ? row + 1 : n;
     const T* mr = M + (long long)row * npad;
-    auto at = [&](int j) { return v[LOWER ? order[j] : j]; };
-    T* const dst = y + (LOWER ? row : order[row]);
-    if constexpr (std::is_same<T, float>::value) {
-        float s[2] = {0.0f, 0.0f}, c[2] = {0.0f, 0.0f};   // two chains
-        auto add = [&](int q, float a, float b) {
+    T s = T(0);
+    [[maybe_unused]] float c = 0.0f;
+    auto add = [&](T a, T b) {
+        if constexpr (std::is_same<T, float>::value) {
             const float p = __fmul_rn(a, b);
-            c[q] = __fadd_rn(c[q], __fmaf_rn(a, b, -p));
-            two_sum_into(s[q], c[q], p);
-        };
-        int j = j0 + lane;
-        for (; j + 224 < j1; j += 256) {   // eight loads of each in flight
-            float a[8], b[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                a[q] = mr[j + 32 * q];
-                b[q] = at(j + 32 * q);
-            }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) add(q & 1, a[q], b[q]);
+            c = __fadd_rn(c, __fmaf_rn(a, b, -p));
+            two_sum_into(s, c, p);
+        } else {
+            s = fma(a, b, s);
         }
-        for (; j < j1; j += 32) add(0, mr[j], at(j));
-        c[0] += c[1];
-        two_sum_into(s[0], c[0], s[1]);
-        for (int o = 16; o > 0; o >>= 1) {
-            const float so = __shfl_xor_sync(0xffffffffu, s[0], o), co = __shfl_xor_sync(0xffffffffu, c[0], o);
-            c[0] += co;
-            two_sum_into(s[0], c[0], so);
-        }
-        if (lane == 0) *dst = s[0] + c[0];
-    } else {
-        double s[2] = {0.0, 0.0};
-        int j = j0 + lane;
-        for (; j + 224 < j1; j += 256) {
-            double a[8], b[8];
+    };
+    constexpr int U = 8;   // loads of each array in flight
+    for (int j = (LOWER ? 0 : row) + tid; j < j1; j += U * kGemv) {
+        T a[U], b[U];
+        int at[U];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                a[q] = mr[j + 32 * q];
-                b[q] = at(j + 32 * q);
-            }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) s[q & 1] = fma(a[q], b[q], s[q & 1]);
+        for (int q = 0; q < U; ++q) {
+            const int jq = j + q * kGemv;
+            a[q] = jq < j1 ? mr[jq] : T(0);
+            at[q] = jq < j1 ? (LOWER ? order[jq] : jq) : -1;
         }
-        for (; j < j1; j += 32) s[0] = fma(mr[j], at(j), s[0]);
-        const double t = warp_sum(s[0] + s[1]);
-        if (lane == 0) *dst = t;
+#pragma unroll
+        for (int q = 0; q < U; ++q) b[q] = at[q] >= 0 ? v[at[q]] : T(0);
+#pragma unroll
+        for (int q = 0; q < U; ++q)
+            if (at[q] >= 0) add(a[q], b[q]);
+    }
+    auto merge = [&](T so, [[maybe_unused]] float co) {
+        if constexpr (std::is_same<T, float>::value) {
+            c += co;
+            two_sum_into(s, c, so);
+        } else {
+            s += so;
+        }
+    };
+    for (int o = 16; o > 0; o >>= 1) {
+        const T so = __shfl_xor_sync(0xffffffffu, s, o);
+        float co = 0.0f;
+        if constexpr (std::is_same<T, float>::value) co = __shfl_xor_sync(0xffffffffu, c, o);
+        merge(so, co);
+    }
+    if (lane == 0) {
+        red[0][w] = s;
+        red[1][w] = (T)c;
+    }
+    __syncthreads();
+    if (tid == 0) {
+#pragma unroll
+        for (int q = 1; q < kGemv / 32; ++q) merge(red[0][q], (float)red[1][q]);
+        y[LOWER ? row : order[row]] = s + (T)c;
     }
 }
 
@@ -590,41 +597,44 @@ void fill(const Ctx& c, long long n, double* v, double value) {
 // below the diagonal block of block column kb: block rows kb+1 .. kb+bb.
 inline int band_blocks(int band) { return (band + TB - 1) / TB; }
 
-void chol_factor(const Ctx& c, double* A, int npad, int band, int* info, double* Dk) {
+void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A, double* W, int npad, int band, int* info,
+                  double* Dk) {
     // the Cholesky factor of a banded matrix keeps its band, so the panel and
     // the trailing update of step kb touch only the bb block rows below it;
-    // the blocks left out are zero in A and L alike
+    // the blocks left out are zero in A and L alike.  W = L^-1 is dense lower
+    // triangular; L_ib,kb vanishes beyond the band, so the update after block
+    // row kb reaches only the bb block rows below.
     const int nb = npad / TB, bb = band_blocks(band);
+    const long long n2 = (long long)npad * npad;
+    const Ctx cs{side, c.launches};
+    auto follow = [&](cudaStream_t from, cudaStream_t to) {   // to waits for what from has been given so far
+        if (side == c.s) return;
+        cudaEventRecord(ready, from);
+        cudaStreamWaitEvent(to, ready, 0);
+    };
     cudaMemsetAsync(info, 0, sizeof(int), c.s);
+    follow(c.s, side);
+    k_identity<<<grid_for(n2, 256), 256, 0, cs.s>>>(W, npad);
+    TOPO_LAUNCH_CHECK(cs);
     for (int kb = 0; kb < nb; ++kb) {
+        const int m = std::min(nb - kb - 1, bb);
         k_potrf_diag<<<1, 512, 0, c.s>>>(A, npad, kb, info, Dk);
         TOPO_LAUNCH_CHECK(c);
-        const int m = std::min(nb - kb - 1, bb);
         if (m > 0) {
             k_trsm_panel<<<dim3(TB / kStrip, m), dim3(TB, kStrip), 0, c.s>>>(A, npad, kb, Dk);
             TOPO_LAUNCH_CHECK(c);
+        }
+        follow(c.s, side);   // block column kb of L and its Dk are final
+        k_trsm_rows<<<dim3(TB / kStrip, kb + 1), dim3(kStrip, TB), 0, cs.s>>>(W, npad, kb, Dk);
+        TOPO_LAUNCH_CHECK(cs);
+        if (m > 0) {
+            k_gemm_update<<<dim3(TB / kStrip, kb + 1, m), dim3(TB, kStrip), 0, cs.s>>>(A, W, npad, kb);
+            TOPO_LAUNCH_CHECK(cs);
             k_syrk<<<dim3(TB / kStrip, m * (m + 1) / 2), dim3(TB, kStrip), 0, c.s>>>(A, npad, kb);
             TOPO_LAUNCH_CHECK(c);
         }
     }
-}
-
-void tri_inverse(const Ctx& c, const double* L, double* W, int npad, int band, const double* Dk) {
-    // W = L^-1 is dense lower triangular; L_ib,kb vanishes beyond the band,
-    // so the update after block row kb reaches only the bb block rows below
-    const int nb = npad / TB, bb = band_blocks(band);
-    const long long n2 = (long long)npad * npad;
-    k_identity<<<grid_for(n2, 256), 256, 0, c.s>>>(W, npad);
-    TOPO_LAUNCH_CHECK(c);
-    for (int kb = 0; kb < nb; ++kb) {
-        k_trsm_rows<<<dim3(TB / kStrip, kb + 1), dim3(kStrip, TB), 0, c.s>>>(W, npad, kb, Dk);
-        TOPO_LAUNCH_CHECK(c);
-        const int m = std::min(nb - kb - 1, bb);
-        if (m > 0) {
-            k_gemm_update<<<dim3(TB / kStrip, kb + 1, m), dim3(TB, kStrip), 0, c.s>>>(L, W, npad, kb);
-            TOPO_LAUNCH_CHECK(c);
-        }
-    }
+    follow(side, c.s);
 }
 
 void transpose_dense(const Ctx& c, const double* W, double* WT, int npad) {
@@ -636,10 +646,9 @@ void transpose_dense(const Ctx& c, const double* W, double* WT, int npad) {
 template <typename T>
 void coarse_apply(const Ctx& c, const Coarse& cs, const T* W, const T* WT, const T* rhs, T* y, T* out) {
     const int n = cs.n, npad = cs.npad;
-    const unsigned blocks = (unsigned)((n + 3) / 4);   // four rows a block: small grids on all SMs
-    k_trigemv<T, true><<<blocks, 128, 0, c.s>>>(n, npad, W, rhs, y, cs.order);
+    k_trigemv<T, true><<<n, kGemv, 0, c.s>>>(n, npad, W, rhs, y, cs.order);
     TOPO_LAUNCH_CHECK(c);
-    k_trigemv<T, false><<<blocks, 128, 0, c.s>>>(n, npad, WT, y, out, cs.order);
+    k_trigemv<T, false><<<n, kGemv, 0, c.s>>>(n, npad, WT, y, out, cs.order);
     TOPO_LAUNCH_CHECK(c);
 }
 template void coarse_apply<double>(const Ctx&, const Coarse&, const double*, const double*, const double*, double*,

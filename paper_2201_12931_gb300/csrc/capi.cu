@@ -184,7 +184,10 @@ void free_all(topo_grid* h) {
     h->mk32 = nullptr;
     h->mkdf = nullptr;
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
-    h->cap_stream = nullptr;
+    if (h->side_stream) cudaStreamDestroy(h->side_stream);
+    if (h->side_event) cudaEventDestroy(h->side_event);
+    h->cap_stream = h->side_stream = nullptr;
+    h->side_event = nullptr;
     for (int q = 0; q < kDirRing; ++q) {
         if (h->graph64[q].exec) cudaGraphExecDestroy(h->graph64[q].exec);
         if (h->graph32[q].exec) cudaGraphExecDestroy(h->graph32[q].exec);
@@ -228,15 +231,25 @@ topo_status ensure_coarse(topo_grid* h) {
         const Ctx cc = h->ctx();
         assemble_coarse(cc, lc.g, h->K0d, lc.E64, h->prm.homogenize == 2 && h->L > 1 ? lc.Ke64 : nullptr, lc.mask,
                         cs.A, cs.npad, cs.order);
-        chol_factor(cc, cs.A, cs.npad, band, cs.info, cs.Dk);
-        tri_inverse(cc, cs.A, cs.W64, cs.npad, band, cs.Dk);
+        const bool fork = cc.s == h->cap_stream && h->side_stream && h->side_event;   // capturing
+        chol_inverse(cc, fork ? h->side_stream : cc.s, h->side_event, cs.A, cs.W64, cs.npad, band, cs.info, cs.Dk);
         transpose_dense(cc, cs.W64, cs.WT64, cs.npad);
         const long long n2 = (long long)cs.npad * cs.npad;
         convert<double, float>(cc, n2, cs.W64, cs.W32);
         convert<double, float>(cc, n2, cs.WT64, cs.WT32);
     };
     PcgGraph& gr = h->coarse_graph;
-    if (h->prm.graphs != 0 && !gr.exec && !gr.failed) capture_launches(h, gr, body);
+    if (h->prm.graphs != 0 && !gr.exec && !gr.failed) {
+        if (!h->side_stream && cudaStreamCreateWithFlags(&h->side_stream, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            h->side_stream = nullptr;
+        }
+        if (!h->side_event && cudaEventCreateWithFlags(&h->side_event, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            h->side_event = nullptr;
+        }
+        capture_launches(h, gr, body);
+    }
     if (gr.exec) {
         CK(h, cudaGraphLaunch(gr.exec, h->stream));
         h->launches += gr.launches;

@@ -189,6 +189,8 @@ struct topo_grid {
     topo::PcgGraph graph64[topo::kDirRing], graph32[topo::kDirRing];   // captured PCG iterations per ring slot
     topo::PcgGraph coarse_graph;            // captured coarsest-grid assembly, factorization and inverse
     cudaStream_t cap_stream = nullptr;  // private stream the graphs are captured on
+    cudaStream_t side_stream = nullptr; // second branch of a captured graph
+    cudaEvent_t side_event = nullptr;
     topo_solve_stats stats{};
     std::string err;
     topo::Ctx ctx() { return topo::Ctx{stream, &launches}; }
@@ -342,11 +344,14 @@ template <typename T>
 void zero(const Ctx& c, long long n, T* v);
 void fill(const Ctx& c, long long n, double* v, double value);
 // dense coarse solve
-// band: half-bandwidth of A in entries (npad for a dense matrix); Dk
-// (npad x 32 doubles) receives the inverses of the 32 x 32 diagonal blocks of
-// L, which tri_inverse reads
-void chol_factor(const Ctx& c, double* A, int npad, int band, int* info, double* Dk);
-void tri_inverse(const Ctx& c, const double* L, double* W, int npad, int band, const double* Dk);
+// A = L L^T in place and W = L^-1.  band: half-bandwidth of A in entries (npad
+// for a dense matrix); Dk (npad x 32 doubles) receives the inverses of the
+// 32 x 32 diagonal blocks of L.  The inverse of a block row needs the factor
+// up to its block column only: with side != c.s (stream capture) its launches
+// go to that stream, ordered by the event, beside the chain of diagonal
+// blocks, and are joined at the end.
+void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A, double* W, int npad, int band, int* info,
+                  double* Dk);
 void transpose_dense(const Ctx& c, const double* W, double* WT, int npad);
 template <typename T>
 void coarse_apply(const Ctx& c, const Coarse& cs, const T* W, const T* WT, const T* rhs, T* y, T* out);
