@@ -18,6 +18,17 @@ __device__ __forceinline__ void ld3(const float* p, float* v) {
     v[1] = a.y;
     v[2] = a.z;
 }
+// a slot whose fourth word carries a value of its own
+__device__ __forceinline__ void st4(float* p, const float* v, float w) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], w);
+}
+__device__ __forceinline__ float ld4(const float* p, float* v) {
+    const float4 a = *reinterpret_cast<const float4*>(p);
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = a.z;
+    return a.w;
+}
 __device__ __forceinline__ void st3(double* p, const double* v) {
     *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
     p[2] = v[2];

@@ -48,6 +48,9 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     constexpr bool NEEDD = (MODE == ST_JACOBI || MODE == ST_JACOBI0 || MODE == ST_JACOBI2);
     constexpr bool J2 = (MODE == ST_JACOBI2);   // u1 = omega D^-1 f formed from f: u is not read
     constexpr bool NEEDF = (MODE != ST_APPLY);   // ST_APPLY_P: p_old in the f slots
+    // FP32 sweeps: the column sums of E for the diagonal ride in the padding
+    // word of the contribution slots, which come from the same neighbours
+    constexpr bool kEslot = (MODE == ST_JACOBI) && std::is_same<T, float>::value;
     constexpr bool PUPD = (MODE == ST_APPLY_P);
     constexpr int nU = (TY + 1) * (TX + 1) * 4, nC = 3 * TY * TX * 4, nEs = TY * TX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -82,9 +85,8 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     const int hx = i0 - 1 + hsx, hy = j0 - 1 + hsy;
     const bool halo_ok = has_halo && hx >= 0 && hx < NX && hy >= 0 && hy < NY;
     // 32-bit vector indices (topo_create_grid keeps 3 * nodes below 2^31):
-    // fewer address instructions; the fused K.p keeps 64-bit indices, with
-    // which it needs fewer registers (measured: 32-bit spilled and was slower)
-    using Ix = std::conditional_t<PUPD, long long, int>;
+    // fewer address instructions and registers
+    using Ix = int;
     const Ix nplane = (Ix)NX * NY;
     // nodes outside the grid read the nearest one inside (their elements have
     // modulus 0): no predicates and zero fills around the loads
@@ -249,11 +251,18 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
                 for (int c = 0; c < 3; ++c) mu[c] = ((chm >> c) & 1u) ? T(0) : shv[B & 1][c];
                 st3(U + hoff, mu);
             }
-            st3(Cb + coff, st10);
-            st3(Cb + nC / 3 + coff, st01);
-            st3(Cb + 2 * (nC / 3) + coff, st11);
+            if constexpr (kEslot) {
+                st4(Cb + coff, st10, stE);
+                st4(Cb + nC / 3 + coff, st01, stE);
+                st4(Cb + 2 * (nC / 3) + coff, st11, stE);
+            } else {
+                st3(Cb + coff, st10);
+                st3(Cb + nC / 3 + coff, st01);
+                st3(Cb + 2 * (nC / 3) + coff, st11);
+            }
         }
-        if constexpr (NEEDD && !J2) Eb[ty * TX + tx] = stE;
+        if constexpr (NEEDD && !J2 && !kEslot) Eb[ty * TX + tx] = stE;
+        [[maybe_unused]] const T ownE = stE;
         // start loading plane P + 1 (its slot held plane P - 3, no longer needed)
         if (P + 1 <= kz1) fetch(std::integral_constant<int, SN>{}, P + 1);
         if constexpr (kDF && NEEDF) {
@@ -268,11 +277,18 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
         const int Q = P - 2;
         if (out_ok && Q >= kz0 && Q < kz1) {
             T y[3] = {T(0), T(0), T(0)};
+            [[maybe_unused]] T sumE = T(0);
             if (NEEDU) {
                 T a0[3], a1[3], a2[3];
-                ld3(Cb + coff - 4, a0);
-                ld3(Cb + nC / 3 + coff - TX * 4, a1);
-                ld3(Cb + 2 * (nC / 3) + coff - TX * 4 - 4, a2);
+                if constexpr (kEslot) {
+                    sumE = ownE + ld4(Cb + coff - 4, a0);
+                    sumE += ld4(Cb + nC / 3 + coff - TX * 4, a1);
+                    sumE += ld4(Cb + 2 * (nC / 3) + coff - TX * 4 - 4, a2);
+                } else {
+                    ld3(Cb + coff - 4, a0);
+                    ld3(Cb + nC / 3 + coff - TX * 4, a1);
+                    ld3(Cb + 2 * (nC / 3) + coff - TX * 4 - 4, a2);
+                }
                 if constexpr (kDF) {   // x and y in paired form (the same operations)
                     st2(y, add2(add2(add2(ld2(st00), ld2(a0)), ld2(a1)), ld2(a2)));
                     y[2] = st00[2] + a0[2] + a1[2] + a2[2];
@@ -287,8 +303,11 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
             if constexpr (J2) {
                 rD = sdv[SO];
             } else if constexpr (NEEDD) {
-                const T* e = Eb + ty * TX + tx;
-                rD = recip(mk.kdiag * (e[0] + e[-1] + e[-TX] + e[-TX - 1]));
+                if constexpr (!kEslot) {
+                    const T* e = Eb + ty * TX + tx;
+                    sumE = e[0] + e[-1] + e[-TX] + e[-TX - 1];
+                }
+                rD = recip(mk.kdiag * sumE);
             }
             TO* o = out + 3 * ((Ix)Q * nplane) + own3;
             const unsigned m2 = sm[SO];
