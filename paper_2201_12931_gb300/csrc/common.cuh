@@ -253,6 +253,9 @@ long long brick_ctas(const Geom& g);
 int brick_apply(const Ctx& c, int mode, const Geom& g, const ModalK<float>& mk, const float* E, const uint8_t* mask,
                 const float* u, const float* f, float* out, float omega, double* dot_partials, const float* Dinv,
                 float* pout, const double* beta, const float* ec, const uint8_t* maskc, const DotTail& tail);
+// fc = diag(free_c) P^T diag(free) (f - K u), on the next coarser level
+void brick_restrict(const Ctx& c, const Geom& g, const ModalK<float>& mk, const float* E, const uint8_t* mask,
+                    const float* u, const float* f, const uint8_t* maskc, float* fc);
 // ---- tc_op.cu: FP32 operators with the element products on tcgen05 tensor cores
 OpLaunch op_launch(const Geom& g, int ty, int target_ctas, int resident_ctas);
 OpLaunch op_launch_tc(const Geom& g, int nsm);

@@ -110,9 +110,9 @@ template int op_apply<double>(topo_grid*, int, int, const double*, const double*
 template int op_apply<float>(topo_grid*, int, int, const float*, const float*, float*, double*, float*,
                              const double*, const float*, const DotTail&);
 
-// whether a Jacobi sweep of level l takes the coarse correction along (op_apply's ec)
+// whether the transfers of level l run inside its operators (op_brick.cu)
 template <typename T>
-static bool fuse_prolong(const topo_grid* h, int l) {
+static bool fuse_transfers(const topo_grid* h, int l) {
     return std::is_same<T, float>::value && h->lev[l].brick && h->prm.tensor_cores == 0 &&
            !(h->prm.homogenize == 2 && l > 0);
 }
@@ -131,6 +131,7 @@ int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot, const D
     T* cur = (nflip & 1) ? tmp : out;
     T* oth = (cur == out) ? tmp : out;
     const long long n = 3 * lv.g.nn;
+    bool restricted = false;
     if (pre > 0) {
         // the first two sweeps from zero as one kernel on matrix-free levels
         const bool two = pre >= 2 && !(h->prm.homogenize == 2 && l > 0);
@@ -144,16 +145,20 @@ int vcycle(topo_grid* h, int l, const T* f, T* out, T* tmp, double* dot, const D
             op_apply<T>(h, ST_JACOBI, l, cur, f, oth, nullptr);
             T* t = cur; cur = oth; oth = t;
         }
-        op_apply<T>(h, ST_RESID, l, cur, f, oth, nullptr);
+        // (while launches are timed, the fine residual is a launch of its own)
+        restricted = fuse_transfers<T>(h, l) && !(h->prof_on && l == 0);
+        if (!restricted) op_apply<T>(h, ST_RESID, l, cur, f, oth, nullptr);
     } else {
         zero<T>(c, n, cur);
         cudaMemcpyAsync(oth, f, sizeof(T) * n, cudaMemcpyDeviceToDevice, h->stream);
     }
     Level& lc = h->lev[l + 1];
     VBuf<T>& vc = P<T>::vb(lc);
-    restrict_residual<T>(c, lv.g, lv.mask, lc.mask, oth, vc.f);
+    if (!restricted) restrict_residual<T>(c, lv.g, lv.mask, lc.mask, oth, vc.f);
+    if constexpr (std::is_same<T, float>::value)
+        if (restricted) brick_restrict(c, lv.g, *h->mk32, lv.E32, lv.mask, cur, f, lc.mask, vc.f);
     vcycle<T>(h, l + 1, vc.f, vc.a, vc.b, nullptr);
-    const T* ec = post > 0 && fuse_prolong<T>(h, l) ? vc.a : nullptr;
+    const T* ec = post > 0 && fuse_transfers<T>(h, l) ? vc.a : nullptr;
     if (!ec) prolong_add<T>(c, lv.g, lv.mask, lc.mask, vc.a, cur);
     int np = 0;
     for (int s = 0; s < post; ++s) {

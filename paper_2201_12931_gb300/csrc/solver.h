@@ -6,7 +6,7 @@
 
 namespace topo {
 // returns the number of dot partials written (0 without dot, -1: reduced and
-// the tail done); ec (JACOBI on levels that fuse_prolong): the iterate is
+// the tail done); ec (JACOBI on levels that fuse_transfers): the iterate is
 // u + P~ ec, ec on level l + 1
 template <typename T>
 int op_apply(topo_grid* h, int mode, int l, const T* u, const T* f, T* out, double* dot, T* pout = nullptr,

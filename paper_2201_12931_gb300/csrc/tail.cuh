@@ -51,10 +51,11 @@ __device__ __forceinline__ void dot_tail(const DotTail& t, const double* partial
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((tid & 31) == 0) red[tid >> 5] = s;
     __syncthreads();
+    if (tid >= 32) return;
+    static_assert(THREADS / 32 <= 16, "one half-warp holds the warps' sums");
+    s = tid < THREADS / 32 ? red[tid] : 0.0;
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (tid == 0) {
-        s = red[0];
-#pragma unroll
-        for (int w = 1; w < THREADS / 32; ++w) s += red[w];
         cg_scalar(t.kind, s, t.sc, t.hist);
         *t.ticket = 0;
     }
