@@ -257,7 +257,7 @@ int brick_apply(const Ctx& c, int mode, const Geom& g, const ModalK<float>& mk, 
 void brick_restrict(const Ctx& c, const Geom& g, const ModalK<float>& mk, const float* E, const uint8_t* mask,
                     const float* u, const float* f, const uint8_t* maskc, float* fc);
 // ---- tc_op.cu: FP32 operators with the element products on tcgen05 tensor cores
-OpLaunch op_launch(const Geom& g, int ty, int target_ctas, int resident_ctas);
+OpLaunch op_launch(const Geom& g, int ty, int resident_ctas);
 OpLaunch op_launch_tc(const Geom& g, int nsm);
 constexpr int kTcBWords = 2304;
 // host: shared-memory image of B = [K0_hi | K0_lo | K0_hi] (TF32), kTcBWords words

@@ -640,49 +640,41 @@ __global__ void __launch_bounds__(256) k_energy_sens_z(ModalCoef mc, const doubl
 
 // Launch geometry: x-y tiles of (kOpTX - 1) x (ty - 1) output node columns
 // and z chunks.  A chunk of cz planes marches over cz + 3 of them, in groups
-// of four (kernels count the groups from the chunk's first plane).  At least
-// target_ctas CTAs where the grid allows; beyond that the number of chunks
-// minimises (waves of resident CTAs) x (steps per CTA), so that neither a
-// nearly empty last wave nor a nearly empty last group costs a whole one:
-// 128x64x64 elements take chunks of 5 planes (8 steps) instead of 4 (12
-// steps while groups began at multiples of four).
-OpLaunch op_launch(const Geom& g, int ty, int target_ctas, int resident_ctas) {
+// of four (kernels count the groups from the chunk's first plane).  The number
+// of chunks minimises (waves of resident CTAs) x (steps per CTA), so that
+// neither a nearly empty last wave nor a nearly empty last group costs a whole
+// one: a grid whose tiles and chunks fit one wave takes long chunks rather
+// than many short ones, each of which marches over three planes more
+// (128x64x64 elements: 250 CTAs of 16 steps, not 650 of 8 in three waves; a
+// V-cycle over 128x64x64 elements 212 -> 196 us, double-FP32 operators of
+// 95x61x43 elements 322 -> 296 us, against at least 1216 CTAs wherever chunks
+// of four planes allow them).
+OpLaunch op_launch(const Geom& g, int ty, int resident_ctas) {
     OpLaunch L;
     L.g = g;
     L.gx = (g.nx + 1 + kOpTX - 2) / (kOpTX - 1);
     L.gy = (g.ny + 1 + ty - 2) / (ty - 1);
     const long long xy = (long long)L.gx * L.gy;
     const int NZ = g.nz + 1;
-    const long long gz_min = (target_ctas + xy - 1) / xy;
-    // chunks of at least 4 planes (each chunk re-reads 3 planes): small
-    // levels get many short chunks, as their launches are bound by the
-    // latency of the march, not by memory
-    constexpr int kMinCz = 4;
-    auto chunk = [&](long long gz) {
-        int cz = (int)((NZ + gz - 1) / gz);
-        return cz < kMinCz ? (NZ < kMinCz ? NZ : kMinCz) : cz;
-    };
-    int best_cz = chunk(gz_min);
-    double best_cost = -1.0;
-    for (long long gz = gz_min; gz <= 8 * gz_min; ++gz) {
-        const int cz = chunk(gz);
-        const long long gz_eff = (NZ + cz - 1) / cz;
-        const long long waves = (xy * gz_eff + resident_ctas - 1) / resident_ctas;
+    double best = -1.0;
+    for (int gz = 1; gz <= std::min(NZ, 16384); ++gz) {   // (the grid's z limit is 65535)
+        const int cz = std::max((NZ + gz - 1) / gz, std::min(4, NZ));   // at least 4 planes
+        const long long chunks = (NZ + cz - 1) / cz;
+        const long long waves = (xy * chunks + resident_ctas - 1) / resident_ctas;
         const double cost = (double)waves * ((cz + 6) / 4 * 4 + 1.5);
-        if (best_cost < 0.0 || cost < best_cost) {
-            best_cost = cost;
-            best_cz = cz;
+        if (best < 0.0 || cost < best) {
+            best = cost;
+            L.cz = cz;
+            L.gz = (int)chunks;
         }
-        if (cz <= kMinCz) break;   // chunks cannot get shorter
+        if (cz <= 4) break;   // chunks cannot get shorter
     }
-    L.cz = best_cz;
-    L.gz = (NZ + best_cz - 1) / best_cz;
     return L;
 }
 
 // resident CTAs per SM: 2 for the FP32 kernel (launch bounds 256 x 2), 1 for FP64
-OpLaunch op_launch32(const Geom& g, int nsm) { return op_launch(g, op_ty<float>(), 1216, 2 * nsm); }
-OpLaunch op_launch64(const Geom& g, int nsm) { return op_launch(g, op_ty<double>(), 608, nsm); }
+OpLaunch op_launch32(const Geom& g, int nsm) { return op_launch(g, op_ty<float>(), 2 * nsm); }
+OpLaunch op_launch64(const Geom& g, int nsm) { return op_launch(g, op_ty<double>(), nsm); }
 
 template <typename T>
 int stencil(const Ctx& c, int mode, const OpLaunch& L, const ModalK<T>& mk, const T* E, const uint8_t* mask,

@@ -427,7 +427,7 @@ void launch_tc(const Ctx& c, const OpLaunch& L, float kdiag, const float* E, con
 
 }  // namespace
 
-OpLaunch op_launch_tc(const Geom& g, int nsm) { return op_launch(g, kTcTY, 2 * nsm, nsm); }
+OpLaunch op_launch_tc(const Geom& g, int nsm) { return op_launch(g, kTcTY, nsm); }
 
 int stencil_tc(const Ctx& c, int mode, const OpLaunch& L, float kdiag, const float* E, const uint8_t* mask,
                const float* u, const float* f, float* out, float omega, const uint32_t* Bimg, double* dot,
