@@ -63,10 +63,10 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     // it leaves only the z-difference of the mean mode, which is added back
     // (4 (ref_P - ref_{P-1}) in element_modal).  Thread 0 keeps the last
     // reference (sref_last) and publishes the split correction of each plane
-    // in a ring of four slots (szc).
+    // in one of two slots (szc).
     constexpr bool kDF = std::is_same<T, dfl>::value;
     __shared__ double sref_last[4];
-    __shared__ __align__(16) float szc[4][8];
+    __shared__ __align__(16) float szc[2][8];
     if (kDF && threadIdx.x == 0 && threadIdx.y == 0) sref_last[0] = sref_last[1] = sref_last[2] = 0.0;
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
@@ -111,8 +111,15 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     // splits them where they are used (a load is never consumed in the step
     // that issues it), and fetches f only one step ahead of its use.
     using TSl = std::conditional_t<kDF, double, T>;
-    TSl su[4][3], sf[4][3], sE[4];
-    unsigned sm[4];
+    // Double-FP32 steps are unrolled by two, not four: four of them overflow
+    // the instruction cache (product, residual and norm over 151x77x93 elements
+    // 296 -> 261 us).  Two slots; the masks of planes P - 1 and P - 2 move down
+    // each step.
+    constexpr int NS = kDF ? 2 : 4, SM = NS - 1;
+    TSl su[NS][3], sf[NS][3], sE[NS];
+    unsigned sm[NS];
+    static_assert(!kDF || !NEEDD, "a sweep reads E of plane P - 1 after the next plane's load: three slots");
+    [[maybe_unused]] unsigned mh[3] = {0u, 0u, 0u};   // (double-FP32) masks of planes P, P - 1, P - 2
     TSl shv[2][3];
     [[maybe_unused]] T shf[2][3] = {};        // halo p_old (ST_APPLY_P) or halo f (ST_JACOBI2)
     [[maybe_unused]] T sdv[4] = {};           // own node D^-1 per plane slot (ST_JACOBI2)
@@ -121,7 +128,7 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     unsigned shm[2];
     [[maybe_unused]] double srf[2][3];   // plane references (double-FP32)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < NS; ++q) {
         su[q][0] = su[q][1] = su[q][2] = TSl(0);
         sf[q][0] = sf[q][1] = sf[q][2] = TSl(0);
         sE[q] = TSl(0);
@@ -190,16 +197,19 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     auto step = [&](auto Bc, int P) {
         constexpr int B = decltype(Bc)::value;
         constexpr int B2 = B & 1;                 // shared-memory buffer
-        constexpr int SN = (B + 1) & 3;           // slot of plane P + 1
-        constexpr int SO = (B + 2) & 3;           // slot of plane P - 2 (output)
-        [[maybe_unused]] constexpr int SL = (B + 3) & 3;   // slot of plane P - 1
+        constexpr int SN = (B + 1) & SM;          // slot of plane P + 1
+        constexpr int SO = (B + 2) & SM;          // slot of plane P - 2 (output)
+        [[maybe_unused]] constexpr int SL = (B + 3) & SM;  // slot of plane P - 1
         T* const U = reinterpret_cast<T*>(smem_raw) + B2 * nU;
         T* const Cb = reinterpret_cast<T*>(smem_raw) + 2 * nU + B2 * nC;
         [[maybe_unused]] T* const Eb = reinterpret_cast<T*>(smem_raw) + 2 * nU + 2 * nC + B2 * nEs;
         // publish plane P (masked) and the stashed contributions of plane P - 2
         if constexpr (kDF) {
             // masked, shifted by the plane reference in FP64, then split
-            const unsigned cm = sm[B];
+            mh[2] = mh[1];
+            mh[1] = mh[0];
+            mh[0] = sm[B];
+            const unsigned cm = mh[0];
             T mu[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) mu[c] = T((((cm >> c) & 1u) ? 0.0 : su[B][c]) - srf[B & 1][c]);
@@ -310,7 +320,7 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
                 rD = recip(mk.kdiag * sumE);
             }
             TO* o = out + 3 * ((Ix)Q * nplane) + own3;
-            const unsigned m2 = sm[SO];
+            const unsigned m2 = kDF ? mh[2] : sm[SO];
             typename DotAcc<T>::type d32 = 0;
             T r[3];
             [[maybe_unused]] T uo[3], fo[3];
@@ -411,16 +421,18 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     using S1 = std::integral_constant<int, 1>;
     using S2 = std::integral_constant<int, 2>;
     using S3 = std::integral_constant<int, 3>;
-    // planes kz0-1 .. kz1+1 in groups of four, the slots counted from the first
+    // planes kz0-1 .. kz1+1 in groups of NS, the slots counted from the first
     // one (the steps past the last are guarded no-ops; op_launch favours chunks
     // without them)
     const int Pfirst = kz0 - 1;
     fetch(S0{}, Pfirst);
-    for (int P = Pfirst; P <= kz1 + 1; P += 4) {
+    for (int P = Pfirst; P <= kz1 + 1; P += NS) {
         step(S0{}, P);
         step(S1{}, P + 1);
-        step(S2{}, P + 2);
-        step(S3{}, P + 3);
+        if constexpr (NS == 4) {
+            step(S2{}, P + 2);
+            step(S3{}, P + 3);
+        }
     }
     if (DOT) {
         double v = (kDF || std::is_same<T, float>::value) ? (double)dotf : dot;
@@ -647,7 +659,7 @@ __global__ void __launch_bounds__(256) k_energy_sens_z(ModalCoef mc, const doubl
 // than many short ones, each of which marches over three planes more
 // (128x64x64 elements: 250 CTAs of 16 steps, not 650 of 8 in three waves; a
 // V-cycle over 128x64x64 elements 212 -> 196 us, double-FP32 operators of
-// 95x61x43 elements 322 -> 296 us, against at least 1216 CTAs wherever chunks
+// 151x77x93 elements 322 -> 296 us, against at least 1216 CTAs wherever chunks
 // of four planes allow them).
 OpLaunch op_launch(const Geom& g, int ty, int resident_ctas) {
     OpLaunch L;
