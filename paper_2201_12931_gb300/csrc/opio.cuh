@@ -4,6 +4,7 @@
 
 #include "common.cuh"
 #include "dfloat.cuh"
+#include "fp64.cuh"
 
 namespace topo {
 
@@ -39,17 +40,19 @@ __device__ __forceinline__ void ld3(const double* p, double* v) {
     v[1] = a.y;
     v[2] = p[2];
 }
+// double-FP32: the high words of x and y, then their low words, as the paired
+// instructions take them from the registers of a 128-bit load
 __device__ __forceinline__ void st3(dfl* p, const dfl* v) {
     float* q = reinterpret_cast<float*>(p);
-    *reinterpret_cast<float4*>(q) = make_float4(v[0].h, v[0].l, v[1].h, v[1].l);
+    *reinterpret_cast<float4*>(q) = make_float4(v[0].h, v[1].h, v[0].l, v[1].l);
     *reinterpret_cast<float2*>(q + 4) = make_float2(v[2].h, v[2].l);
 }
 __device__ __forceinline__ void ld3(const dfl* p, dfl* v) {
     const float* q = reinterpret_cast<const float*>(p);
     const float4 a = *reinterpret_cast<const float4*>(q);
     const float2 b = *reinterpret_cast<const float2*>(q + 4);
-    v[0] = dfl(a.x, a.y);
-    v[1] = dfl(a.z, a.w);
+    v[0] = dfl(a.x, a.z);
+    v[1] = dfl(a.y, a.w);
     v[2] = dfl(b.x, b.y);
 }
 // vector element loads / stores with widening from and rounding to the
@@ -60,7 +63,8 @@ __device__ __forceinline__ float ldv(const bf16* p) { return __bfloat162float(*p
 __device__ __forceinline__ void stv(float* p, float v) { *p = v; }
 __device__ __forceinline__ void stv(double* p, double v) { *p = v; }
 __device__ __forceinline__ void stv(bf16* p, float v) { *p = __float2bfloat16_rn(v); }
-__device__ __forceinline__ void stv(double* p, dfl v) { *p = df_to_double(v); }
+// (the words widened on the integer pipe: one FP64 instruction instead of three)
+__device__ __forceinline__ void stv(double* p, dfl v) { *p = widen(v.h) + widen(v.l); }
 __device__ __forceinline__ void stv(float* p, dfl v) { *p = df_to_float(v); }
 // per-thread accumulator of the fused dot products
 template <typename T>

@@ -61,13 +61,18 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     // tile rather than its absolute size.  K annihilates a translation, and
     // within a plane the shift is one; between the two planes of an element
     // it leaves only the z-difference of the mean mode, which is added back
-    // (4 (ref_P - ref_{P-1}) in element_modal).  Thread 0 keeps the last
-    // reference (sref_last) and publishes the split correction of each plane
-    // in one of two slots (szc).
+    // (4 (ref_P - ref_{P-1}) in element_modal).  Three lanes of the last warp
+    // (the first two have the halo nodes' FP64 differences) keep the last
+    // reference (sref_last) and publish the split correction of each plane in
+    // one of two slots (szc).  FP64 instructions are what a warp waits for
+    // here, 64 clocks each: with results widened on the integer pipe and the
+    // high words of x and y side by side in shared memory, product and
+    // residual over 151x77x93 elements went from 261 to 239 us.
     constexpr bool kDF = std::is_same<T, dfl>::value;
     __shared__ double sref_last[4];
     __shared__ __align__(16) float szc[2][8];
-    if (kDF && threadIdx.x == 0 && threadIdx.y == 0) sref_last[0] = sref_last[1] = sref_last[2] = 0.0;
+    const bool zc_lane = threadIdx.y == op_ty<T>() - 1 && threadIdx.x < 3;
+    if (kDF && zc_lane) sref_last[threadIdx.x] = 0.0;
 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int NX = nx + 1, NY = ny + 1;
@@ -112,7 +117,7 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     // that issues it), and fetches f only one step ahead of its use.
     using TSl = std::conditional_t<kDF, double, T>;
     // Double-FP32 steps are unrolled by two, not four: four of them overflow
-    // the instruction cache (product, residual and norm over 151x77x93 elements
+    // the instruction cache (product and residual over 151x77x93 elements
     // 296 -> 261 us).  Two slots; the masks of planes P - 1 and P - 2 move down
     // each step.
     constexpr int NS = kDF ? 2 : 4, SM = NS - 1;
@@ -213,14 +218,12 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
             T mu[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) mu[c] = T((((cm >> c) & 1u) ? 0.0 : su[B][c]) - srf[B & 1][c]);
-            if (tid == 0) {   // correction of the element between planes P - 1 and P
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const dfl d = df_from_double(srf[B & 1][c] - sref_last[c]);
-                    szc[B][2 * c] = 4.0f * d.h;   // exact: a power of two
-                    szc[B][2 * c + 1] = 4.0f * d.l;
-                    sref_last[c] = srf[B & 1][c];
-                }
+            if (zc_lane) {   // correction of the element between planes P - 1 and P
+                const double ref = tx == 0 ? srf[B & 1][0] : tx == 1 ? srf[B & 1][1] : srf[B & 1][2];
+                const dfl d = df_from_double(ref - sref_last[tx]);
+                szc[B][2 * tx] = 4.0f * d.h;   // exact: a power of two
+                szc[B][2 * tx + 1] = 4.0f * d.l;
+                sref_last[tx] = ref;
             }
             st3(U + uoff, mu);
             if (has_halo) {
