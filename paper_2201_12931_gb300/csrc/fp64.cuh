@@ -39,13 +39,11 @@ __device__ __forceinline__ double widen(float v) {
     if (m == 0u) return __hiloint2double((int)b, 0);
     return (double)v;
 }
-// 1 / b by two Newton steps from the FP32 reciprocal, for 2^-100 <= b < 2^100
-__device__ __forceinline__ double recip_seeded(double b) {
+// the FP32 reciprocal y0 of b, 2^-100 <= b < 2^100: relative error below 2^-21
+__device__ __forceinline__ double recip_seed(double b) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(trunc_f32(b)));
-    double y = widen_f32(r);
-    y = fma(fma(-b, y, 1.0), y, y);
-    return fma(fma(-b, y, 1.0), y, y);
+    return widen_f32(r);
 }
 __device__ __forceinline__ bool seed_range(double b) {
     return (unsigned)((__double2hiint(b) >> 20) - (1023 - 100)) < 200u;
