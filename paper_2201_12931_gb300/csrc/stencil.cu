@@ -425,14 +425,15 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     using S2 = std::integral_constant<int, 2>;
     using S3 = std::integral_constant<int, 3>;
     // planes kz0-1 .. kz1+1 in groups of NS, the slots counted from the first
-    // one (the steps past the last are guarded no-ops; op_launch favours chunks
-    // without them)
+    // one; the march ends after the second step of a group where that is the
+    // last (a step past the last is a guarded no-op)
     const int Pfirst = kz0 - 1;
     fetch(S0{}, Pfirst);
     for (int P = Pfirst; P <= kz1 + 1; P += NS) {
         step(S0{}, P);
         step(S1{}, P + 1);
         if constexpr (NS == 4) {
+            if (P + 2 > kz1 + 1) break;   // (uniform in the CTA)
             step(S2{}, P + 2);
             step(S3{}, P + 3);
         }
@@ -654,16 +655,17 @@ __global__ void __launch_bounds__(256) k_energy_sens_z(ModalCoef mc, const doubl
 }  // namespace
 
 // Launch geometry: x-y tiles of (kOpTX - 1) x (ty - 1) output node columns
-// and z chunks.  A chunk of cz planes marches over cz + 3 of them, in groups
-// of four (kernels count the groups from the chunk's first plane).  The number
-// of chunks minimises (waves of resident CTAs) x (steps per CTA), so that
-// neither a nearly empty last wave nor a nearly empty last group costs a whole
-// one: a grid whose tiles and chunks fit one wave takes long chunks rather
-// than many short ones, each of which marches over three planes more
-// (128x64x64 elements: 250 CTAs of 16 steps, not 650 of 8 in three waves; a
-// V-cycle over 128x64x64 elements 212 -> 196 us, double-FP32 operators of
-// 151x77x93 elements 322 -> 296 us, against at least 1216 CTAs wherever chunks
-// of four planes allow them).
+// and z chunks.  A chunk of cz planes marches over cz + 3 of them, in pairs of
+// steps (counted from the chunk's first plane).  The number of chunks
+// minimises (waves of resident CTAs) x (steps per CTA), so that neither a
+// nearly empty last wave nor a half-used last pair costs a whole one: a grid
+// whose tiles and chunks fit one wave takes long chunks rather than many short
+// ones, each of which marches over three planes more (128x64x64 elements: 300
+// CTAs of 14 steps, not 650 of 8 in three waves).  Measured against at least
+// 1216 CTAs wherever chunks of four planes allow them, then against whole
+// groups of four steps: V-cycle over 128x64x64 elements 212 -> 196 -> 193 us,
+// operators of 256x128x128 elements 561 -> 558 -> 543 us, double-FP32 operators
+// of 151x77x93 elements 322 -> 296 us.
 OpLaunch op_launch(const Geom& g, int ty, int resident_ctas) {
     OpLaunch L;
     L.g = g;
@@ -676,7 +678,7 @@ OpLaunch op_launch(const Geom& g, int ty, int resident_ctas) {
         const int cz = std::max((NZ + gz - 1) / gz, std::min(4, NZ));   // at least 4 planes
         const long long chunks = (NZ + cz - 1) / cz;
         const long long waves = (xy * chunks + resident_ctas - 1) / resident_ctas;
-        const double cost = (double)waves * ((cz + 6) / 4 * 4 + 1.5);
+        const double cost = (double)waves * ((cz + 4) / 2 * 2 + 1.5);
         if (best < 0.0 || cost < best) {
             best = cost;
             L.cz = cz;
