@@ -259,6 +259,16 @@ __global__ void k_axpy_f32(long long n, const float* __restrict__ d, double* __r
 // threads, instead of one tile per CTA.
 constexpr int kStrip = 4;
 
+// One step of the factorization: the diagonal blocks kb of one or two chains
+// that do not touch each other, and the block rows below each that are not
+// zero: m1 of its own chain, then (up to m) separator rows from s0 on.  W has
+// columns c0 .. kb in block row kb.
+struct Front {
+    int chains, kb[2], c0[2], m1[2], s0[2], m[2];
+    __device__ int row(int q, int t) const { return t < m1[q] ? kb[q] + 1 + t : s0[q] + t - m1[q]; }
+    __device__ bool sep(int q, int b) const { return b >= s0[q] && b < s0[q] + m[q] - m1[q]; }
+};
+
 // Cholesky factor of diagonal block kb and its inverse by one CTA, as
 // A = U D U^T (U unit lower) with W = U^-1 carried along, so that a pivot step
 // is a reciprocal, one rank-one update and one barrier.  FP64 instructions
@@ -276,16 +286,17 @@ constexpr int kStrip = 4;
 // the columns spread evenly over 16 warps, one a register, and the warp of the
 // next pivot's column doing that first).
 //
+// One CTA per chain: a step of two chains takes as long as one of one.
 // L goes back to the block (zeros above the diagonal), L^-1 to Dk (block kb:
 // TB x TB row-major at Dk + kb TB^2).  A non-positive or non-finite pivot sets
 // info to its row + 1 (first one wins) and continues with pivot 1.
-__global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int npad, int kb, int* info,
+__global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int npad, Front f, int* info,
                                                     double* __restrict__ Dk) {
     static_assert(TB == 32, "a lane per row");
     __shared__ double col[TB][TB + 1], ucol[TB][TB + 1];   // pivot columns and U's (rows below the diagonal)
     __shared__ double next[2][TB], piv[TB], root[TB];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const long long base = (long long)kb * TB;
+    const long long base = (long long)f.kb[blockIdx.x] * TB;
     const bool worker = w & 3;
     // registers c = cs, cs + 12 of A and W (up to 16; column 0 of A is never
     // updated), this lane's row and column of each
@@ -378,13 +389,16 @@ __global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int 
     }
 }
 
-// L_ib,kb = A_ib,kb L_kk^-T: block row ib = kb+1+blockIdx.y, its rows
-// kStrip*blockIdx.x .. +kStrip (threads: 32 columns x kStrip rows)
-__global__ void __launch_bounds__(128) k_trsm_panel(double* __restrict__ A, int npad, int kb,
+// L_ib,kb = A_ib,kb L_kk^-T: block row ib = row blockIdx.y of chain
+// blockIdx.z, its rows kStrip*blockIdx.x .. +kStrip (threads: 32 columns x
+// kStrip rows)
+__global__ void __launch_bounds__(128) k_trsm_panel(double* __restrict__ A, int npad, Front f,
                                                     const double* __restrict__ Dk) {
     __shared__ double sI[TB][TB + 1];
     __shared__ double sA[kStrip][TB + 1];
-    const int ib = kb + 1 + blockIdx.y, r0 = kStrip * blockIdx.x;
+    const int q = blockIdx.z;
+    if (blockIdx.y >= f.m[q]) return;
+    const int kb = f.kb[q], ib = f.row(q, blockIdx.y), r0 = kStrip * blockIdx.x;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TB + tx;
     const long long rb = (long long)ib * TB + r0, cb = (long long)kb * TB;
     for (int e = tid; e < TB * TB; e += 128) sI[e / TB][e % TB] = Dk[cb * TB + e];
@@ -396,26 +410,37 @@ __global__ void __launch_bounds__(128) k_trsm_panel(double* __restrict__ A, int 
     A[(rb + ty) * npad + cb + tx] = s;
 }
 
-// A_ib,jb -= L_ib,kb L_jb,kb^T for kb < jb <= ib (pair blockIdx.y), rows
-// kStrip*blockIdx.x .. +kStrip of the tile
-__global__ void __launch_bounds__(128) k_syrk(double* __restrict__ A, int npad, int kb) {
+// A_ib,jb -= L_ib,kb L_jb,kb^T for the pairs jb <= ib of a chain's rows (pair
+// blockIdx.y), rows kStrip*blockIdx.x .. +kStrip of the tile.  blockIdx.z: the
+// chain; with two chains, whose separator rows overlap, their pairs of
+// separator rows are left to blockIdx.z = 2, which subtracts both (pairs of
+// the ns rows from sep0 on).
+__global__ void __launch_bounds__(128) k_syrk(double* __restrict__ A, int npad, Front f, int sep0, int ns) {
     __shared__ double sI[kStrip][TB + 1];
     __shared__ double sJ[TB][TB + 1];
-    const int t = blockIdx.y;
+    const int t = blockIdx.y, z = blockIdx.z;
     int ii = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
     while ((ii + 1) * (ii + 2) / 2 <= t) ++ii;
     while (ii * (ii + 1) / 2 > t) --ii;
     const int jj = t - ii * (ii + 1) / 2;
-    const int ib = kb + 1 + ii, jb = kb + 1 + jj, r0 = kStrip * blockIdx.x;
+    if (ii >= (z < 2 ? f.m[z] : ns) || (z < 2 && f.chains == 2 && jj >= f.m1[z])) return;
+    const int ib = z < 2 ? f.row(z, ii) : sep0 + ii, jb = z < 2 ? f.row(z, jj) : sep0 + jj, r0 = kStrip * blockIdx.x;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TB + tx;
-    const long long cb = (long long)kb * TB, rb = (long long)ib * TB + r0, jr = (long long)jb * TB;
-    sI[ty][tx] = A[(rb + ty) * npad + cb + tx];
-    for (int e = tid; e < TB * TB; e += 128) sJ[e / TB][e % TB] = A[(jr + e / TB) * npad + cb + e % TB];
-    __syncthreads();
-    double s = 0.0;
+    const long long rb = (long long)ib * TB + r0, jr = (long long)jb * TB;
+    double v = A[(rb + ty) * npad + jr + tx];
+    for (int q = z < 2 ? z : 0; q < (z < 2 ? z + 1 : 2); ++q) {
+        if (z == 2 && !(f.sep(q, ib) && f.sep(q, jb))) continue;   // (the same for the whole block)
+        const long long cb = (long long)f.kb[q] * TB;
+        __syncthreads();
+        sI[ty][tx] = A[(rb + ty) * npad + cb + tx];
+        for (int e = tid; e < TB * TB; e += 128) sJ[e / TB][e % TB] = A[(jr + e / TB) * npad + cb + e % TB];
+        __syncthreads();
+        double s = 0.0;
 #pragma unroll 8
-    for (int c = 0; c < TB; ++c) s += sI[ty][c] * sJ[tx][c];
-    A[(rb + ty) * npad + jr + tx] -= s;
+        for (int c = 0; c < TB; ++c) s += sI[ty][c] * sJ[tx][c];
+        v -= s;
+    }
+    A[(rb + ty) * npad + jr + tx] = v;
 }
 
 __global__ void k_identity(double* __restrict__ W, int npad) {
@@ -425,13 +450,15 @@ __global__ void k_identity(double* __restrict__ W, int npad) {
     W[i] = ((i / npad) == (i % npad)) ? 1.0 : 0.0;
 }
 
-// W_kb,jb = L_kk^-1 B_kb,jb for jb = blockIdx.y <= kb, its columns
-// kStrip*blockIdx.x .. +kStrip (threads: kStrip columns x 32 rows)
-__global__ void __launch_bounds__(128) k_trsm_rows(double* __restrict__ W, int npad, int kb,
+// W_kb,jb = L_kk^-1 B_kb,jb for jb = c0 + blockIdx.y <= kb of chain
+// blockIdx.z, its columns kStrip*blockIdx.x .. +kStrip (threads: kStrip columns
+// x 32 rows)
+__global__ void __launch_bounds__(128) k_trsm_rows(double* __restrict__ W, int npad, Front f,
                                                    const double* __restrict__ Dk) {
     __shared__ double sI[TB][TB + 1];
     __shared__ double sB[TB][kStrip + 1];
-    const int jb = blockIdx.y, c0 = kStrip * blockIdx.x;
+    const int kb = f.kb[blockIdx.z], jb = f.c0[blockIdx.z] + blockIdx.y, c0 = kStrip * blockIdx.x;
+    if (jb > kb) return;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kStrip + tx;
     const long long rb = (long long)kb * TB, cb = (long long)jb * TB + c0;
     for (int e = tid; e < TB * TB; e += 128) sI[e / TB][e % TB] = Dk[rb * TB + e];
@@ -443,13 +470,16 @@ __global__ void __launch_bounds__(128) k_trsm_rows(double* __restrict__ W, int n
     W[(rb + ty) * npad + cb + tx] = s;
 }
 
-// B_ib,jb -= L_ib,kb W_kb,jb for jb = blockIdx.y <= kb, ib = kb+1+blockIdx.z,
-// rows kStrip*blockIdx.x .. +kStrip of the tile
+// B_ib,jb -= L_ib,kb W_kb,jb for jb = c0 + blockIdx.y <= kb and the rows ib of
+// a chain (blockIdx.z: mm rows of the first chain, then the second's; their
+// columns differ), rows kStrip*blockIdx.x .. +kStrip of the tile
 __global__ void __launch_bounds__(128) k_gemm_update(const double* __restrict__ L, double* __restrict__ W, int npad,
-                                                     int kb) {
+                                                     Front f, int mm) {
     __shared__ double sL[kStrip][TB + 1];
     __shared__ double sW[TB][TB + 1];
-    const int jb = blockIdx.y, ib = kb + 1 + blockIdx.z, r0 = kStrip * blockIdx.x;
+    const int q = blockIdx.z >= mm, i = blockIdx.z - q * mm, kb = f.kb[q], jb = f.c0[q] + blockIdx.y;
+    if (i >= f.m[q] || jb > kb) return;
+    const int ib = f.row(q, i), r0 = kStrip * blockIdx.x;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TB + tx;
     const long long kbase = (long long)kb * TB, rb = (long long)ib * TB + r0, cb = (long long)jb * TB;
     sL[ty][tx] = L[(rb + ty) * npad + kbase + tx];
@@ -643,14 +673,19 @@ void fill(const Ctx& c, long long n, double* v, double value) {
 // below the diagonal block of block column kb: block rows kb+1 .. kb+bb.
 inline int band_blocks(int band) { return (band + TB - 1) / TB; }
 
-void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A, double* W, int npad, int band, int* info,
-                  double* Dk) {
-    // the Cholesky factor of a banded matrix keeps its band, so the panel and
-    // the trailing update of step kb touch only the bb block rows below it;
-    // the blocks left out are zero in A and L alike.  W = L^-1 is dense lower
-    // triangular; L_ib,kb vanishes beyond the band, so the update after block
-    // row kb reaches only the bb block rows below.
-    const int nb = npad / TB, bb = band_blocks(band);
+void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A, double* W, int n, int npad, int band,
+                  int* info, double* Dk) {
+    // The Cholesky factor of a banded matrix keeps its band, so the panel and
+    // the trailing update of a step touch only the bb block rows below it; the
+    // blocks left out are zero in A and L alike.  Two chains of `a` blocks run
+    // to the separator in the same launches (60 steps of 13 x 7 x 7 nodes
+    // become 33: the factorization and inverse of a density update take 1.0 ms
+    // less), then the separator, whose rows keep their order and so their
+    // band.  W = L^-1 is lower triangular with a zero block between the chains;
+    // L_ib,kb vanishes outside a step's rows, so the update after block row kb
+    // reaches only those.
+    const int nb = npad / TB, bb = band_blocks(band), a = coarse_chain(n, band), sep0 = 2 * a, ns = nb - sep0;
+    const int nsep = n - 2 * TB * a;   // rows of the separator
     const long long n2 = (long long)npad * npad;
     const Ctx cs{side, c.launches};
     auto follow = [&](cudaStream_t from, cudaStream_t to) {   // to waits for what from has been given so far
@@ -662,21 +697,43 @@ void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A,
     follow(c.s, side);
     k_identity<<<grid_for(n2, 256), 256, 0, cs.s>>>(W, npad);
     TOPO_LAUNCH_CHECK(cs);
-    for (int kb = 0; kb < nb; ++kb) {
-        const int m = std::min(nb - kb - 1, bb);
-        k_potrf_diag<<<1, 512, 0, c.s>>>(A, npad, kb, info, Dk);
+    for (int step = 0; step < a + ns; ++step) {
+        Front f{};
+        f.chains = step < a ? 2 : 1;
+        if (f.chains == 2) {
+            for (int q = 0; q < 2; ++q) {
+                f.kb[q] = q * a + step;
+                f.c0[q] = q * a;
+                f.m1[q] = std::min(a - 1 - step, bb);
+            }
+            // separator rows in reach: blocks from the front for the first
+            // chain, rows from the back for the second
+            const int front = std::max(0, std::min(ns, step + bb - (a - 1)));
+            const int back = std::max(0, std::min(nsep, TB * (step + 1 - a) + band));
+            f.s0[0] = sep0;
+            f.m[0] = f.m1[0] + front;
+            f.s0[1] = sep0 + (nsep - back) / TB;
+            f.m[1] = f.m1[1] + (back > 0 ? ns - (nsep - back) / TB : 0);
+        } else {
+            f.kb[0] = sep0 + step - a;
+            f.m1[0] = f.m[0] = std::min(nb - f.kb[0] - 1, bb);
+        }
+        const int m = std::max(f.m[0], f.m[1]), cols = f.kb[0] - f.c0[0] + 1, nz = f.chains;
+        const bool sep = f.m[0] > f.m1[0] || f.m[1] > f.m1[1];
+        k_potrf_diag<<<nz, 512, 0, c.s>>>(A, npad, f, info, Dk);
         TOPO_LAUNCH_CHECK(c);
         if (m > 0) {
-            k_trsm_panel<<<dim3(TB / kStrip, m), dim3(TB, kStrip), 0, c.s>>>(A, npad, kb, Dk);
+            k_trsm_panel<<<dim3(TB / kStrip, m, nz), dim3(TB, kStrip), 0, c.s>>>(A, npad, f, Dk);
             TOPO_LAUNCH_CHECK(c);
         }
         follow(c.s, side);   // block column kb of L and its Dk are final
-        k_trsm_rows<<<dim3(TB / kStrip, kb + 1), dim3(kStrip, TB), 0, cs.s>>>(W, npad, kb, Dk);
+        k_trsm_rows<<<dim3(TB / kStrip, cols, nz), dim3(kStrip, TB), 0, cs.s>>>(W, npad, f, Dk);
         TOPO_LAUNCH_CHECK(cs);
         if (m > 0) {
-            k_gemm_update<<<dim3(TB / kStrip, kb + 1, m), dim3(TB, kStrip), 0, cs.s>>>(A, W, npad, kb);
+            k_gemm_update<<<dim3(TB / kStrip, cols, m * nz), dim3(TB, kStrip), 0, cs.s>>>(A, W, npad, f, m);
             TOPO_LAUNCH_CHECK(cs);
-            k_syrk<<<dim3(TB / kStrip, m * (m + 1) / 2), dim3(TB, kStrip), 0, c.s>>>(A, npad, kb);
+            const int pairs = std::max(m * (m + 1) / 2, sep ? ns * (ns + 1) / 2 : 0);
+            k_syrk<<<dim3(TB / kStrip, pairs, sep ? 3 : nz), dim3(TB, kStrip), 0, c.s>>>(A, npad, f, sep0, ns);
             TOPO_LAUNCH_CHECK(c);
         }
     }

@@ -232,7 +232,8 @@ topo_status ensure_coarse(topo_grid* h) {
         assemble_coarse(cc, lc.g, h->K0d, lc.E64, h->prm.homogenize == 2 && h->L > 1 ? lc.Ke64 : nullptr, lc.mask,
                         cs.A, cs.npad, cs.order);
         const bool fork = cc.s == h->cap_stream && h->side_stream && h->side_event;   // capturing
-        chol_inverse(cc, fork ? h->side_stream : cc.s, h->side_event, cs.A, cs.W64, cs.npad, band, cs.info, cs.Dk);
+        chol_inverse(cc, fork ? h->side_stream : cc.s, h->side_event, cs.A, cs.W64, cs.n, cs.npad, band, cs.info,
+                     cs.Dk);
         transpose_dense(cc, cs.W64, cs.WT64, cs.npad);
         const long long n2 = (long long)cs.npad * cs.npad;
         convert<double, float>(cc, n2, cs.W64, cs.W32);

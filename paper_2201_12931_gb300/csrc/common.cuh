@@ -90,7 +90,7 @@ struct Coarse {           // dense coarsest-grid solve: K_c^-1 = W^T W, W = L^-1
     double* y64 = nullptr;    // temporaries of length npad
     float* y32 = nullptr;
     int* info = nullptr;      // device: first non-positive pivot + 1 (0 = ok)
-    int* order = nullptr;     // DOF of the level's node order at each row: nodes run along the shortest axis first
+    int* order = nullptr;     // DOF of the level's node order at each row: nodes along the shortest axis first, then two-ended
     double* Dk = nullptr;     // inverses of the 32 x 32 diagonal blocks of L (npad x 32)
 };
 
@@ -268,13 +268,19 @@ int stencil_tc(const Ctx& c, int mode, const OpLaunch& L, float kdiag, const flo
                const float* u, const float* f, float* out, float omega, const uint32_t* Bimg, double* dot_partials,
                int* err);
 // dense coarsest operator from E_e K0, or from stored element matrices Ke (non-null);
-// order (3 * nodes) receives the DOF of each row
+// order (3 * nodes) receives the DOF of each row (two-ended, see coarse_chain)
 void assemble_coarse(const Ctx& c, const Geom& g, const double* K0, const double* E, const double* Ke,
                      const uint8_t* mask, double* A, int npad, int* order);
 // Half-bandwidth of that operator: rows follow the node order with the
 // shortest axis running fastest and the longest slowest, which makes it
 // 3 (1 + N0 + N0 N1) + 2 for the two smaller node counts N0 <= N1
 int coarse_band(const Geom& g);
+// The factorization is a chain of 32 x 32 diagonal blocks.  A matrix of n rows
+// and half-bandwidth band is eliminated from both ends at once: the first and
+// the last coarse_chain blocks of rows do not touch each other as long as the
+// rows between them are band or more.  Rows are stored in that order: the first
+// t = 32 coarse_chain rows, the last t backwards, then those between.
+inline int coarse_chain(int n, int band) { return n > band ? (n - band) / 64 : 0; }
 // ---- galerkin.cu: stored Galerkin coarse element matrices ------------------
 void galerkin_init_constants();
 // host: the 8 child matrices G_o = P_o^T K0 P_o (8 x 576, o-major)
@@ -347,14 +353,15 @@ template <typename T>
 void zero(const Ctx& c, long long n, T* v);
 void fill(const Ctx& c, long long n, double* v, double value);
 // dense coarse solve
-// A = L L^T in place and W = L^-1.  band: half-bandwidth of A in entries (npad
-// for a dense matrix); Dk (npad x 32 doubles) receives the inverses of the
+// A = L L^T in place and W = L^-1 for n rows in two-ended order (see
+// coarse_chain).  band: half-bandwidth of A in entries before the reordering
+// (npad for a dense matrix); Dk (npad x 32 doubles) receives the inverses of the
 // 32 x 32 diagonal blocks of L.  The inverse of a block row needs the factor
 // up to its block column only: with side != c.s (stream capture) its launches
 // go to that stream, ordered by the event, beside the chain of diagonal
 // blocks, and are joined at the end.
-void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A, double* W, int npad, int band, int* info,
-                  double* Dk);
+void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A, double* W, int n, int npad, int band,
+                  int* info, double* Dk);
 void transpose_dense(const Ctx& c, const double* W, double* WT, int npad);
 template <typename T>
 void coarse_apply(const Ctx& c, const Coarse& cs, const T* W, const T* WT, const T* rhs, T* y, T* out);

@@ -486,10 +486,14 @@ void launch_mode(const Ctx& c, const OpLaunch& L, const ModalK<T>& mk, const T* 
 // node, column component) gathers, in a fixed order, the <= 8 elements that
 // contain both nodes -- element matrices E_e K0, or the stored Ke[e] of a
 // Galerkin level.  Rows and columns of fixed DOFs stay zero here.
-// row of a node's first DOF / 3: nodes numbered along the shortest axis first
+// row of a node's DOF: nodes numbered along the shortest axis first, the first
+// and last t of the n rows eliminated from both ends (coarse_chain)
 struct NodeOrder {
-    int sx, sy, sz;
-    __device__ int at(int i, int j, int k) const { return sx * i + sy * j + sz * k; }
+    int sx, sy, sz, n, t;
+    __device__ int row(int i, int j, int k, int c) const {
+        const int r = 3 * (sx * i + sy * j + sz * k) + c;
+        return r < t ? r : r >= n - t ? t + (n - 1 - r) : t + r;
+    }
 };
 
 __global__ void k_assemble(const double* __restrict__ K0, const double* __restrict__ E,
@@ -521,7 +525,7 @@ __global__ void k_assemble(const double* __restrict__ K0, const double* __restri
                 const int r = 3 * a + c, s = 3 * b + d;
                 v += Ke ? Ke[e * 576 + r * 24 + s] : E[e] * K0[r * 24 + s];
             }
-    A[(3 * no.at(i, j, k) + c) * (long long)npad + 3 * no.at(i2, j2, k2) + d] = v;
+    A[no.row(i, j, k, c) * (long long)npad + no.row(i2, j2, k2, d)] = v;
 }
 
 // unit diagonal of fixed and padding rows, and the DOF of every row
@@ -533,7 +537,7 @@ __global__ void k_assemble_diag(const uint8_t* __restrict__ mask, double* __rest
     int row = d;
     if (d < n) {
         const int node = d / 3;
-        row = 3 * no.at(node % NX, node / NX % NY, node / (NX * NY)) + d % 3;
+        row = no.row(node % NX, node / NX % NY, node / (NX * NY), d % 3);
         order[row] = d;
     }
     if (d >= n || ((mask[d / 3] >> (d % 3)) & 1u)) A[(long long)row * npad + row] = 1.0;
@@ -749,28 +753,27 @@ int stencil_df(const Ctx& c, int mode, const OpLaunch& L, const ModalK<dfl>& mk,
     return dot ? L.gx * L.gy * L.gz : 0;
 }
 
-// strides of the three axes in the row order, and the two smaller node counts
-static NodeOrder node_order(const Geom& g, int* small) {
+// strides of the three axes in the row order, and the half-bandwidth
+static NodeOrder node_order(const Geom& g, int* band) {
     const int N[3] = {g.NX(), g.NY(), g.NZ()};
     int ax[3] = {0, 1, 2}, stride[3];
     std::stable_sort(ax, ax + 3, [&](int a, int b) { return N[a] < N[b]; });
     for (int q = 0, s = 1; q < 3; s *= N[ax[q++]]) stride[ax[q]] = s;
-    if (small) {
-        small[0] = N[ax[0]];
-        small[1] = N[ax[1]];
-    }
-    return NodeOrder{stride[0], stride[1], stride[2]};
+    const int n = 3 * (int)g.nn;   // (at most kMaxCoarseDofs)
+    *band = 3 * (1 + N[ax[0]] + N[ax[0]] * N[ax[1]]) + 2;
+    return NodeOrder{stride[0], stride[1], stride[2], n, 32 * coarse_chain(n, *band)};
 }
 
 int coarse_band(const Geom& g) {
-    int n[2];
-    node_order(g, n);
-    return 3 * (1 + n[0] + n[0] * n[1]) + 2;
+    int band;
+    node_order(g, &band);
+    return band;
 }
 
 void assemble_coarse(const Ctx& c, const Geom& g, const double* K0, const double* E, const double* Ke,
                      const uint8_t* mask, double* A, int npad, int* order) {
-    const NodeOrder no = node_order(g, nullptr);
+    int band;
+    const NodeOrder no = node_order(g, &band);
     cudaMemsetAsync(A, 0, sizeof(double) * (size_t)npad * npad, c.s);
     const long long total = 3 * g.nn * 81;
     k_assemble<<<(unsigned)((total + 255) / 256), 256, 0, c.s>>>(K0, E, Ke, mask, A, g.nx, g.ny, g.nz, npad, no);

@@ -1,8 +1,9 @@
 """Factor and inverse of the coarsest grid by blocks of 32: one level, so that
 the V-cycle is the direct solve, at orders below a block's multiple, on it (96,
-288) and just past it (225), with moduli over nine orders of magnitude.  The
-tolerance is the order times the condition number of the matrix scaled to a unit
-diagonal times 2^-53, from the matrix itself."""
+288) and just past it (225), eliminated from both ends (225 and more) and not,
+with moduli over nine orders of magnitude.  The tolerance is the order times the
+condition number of the matrix scaled to a unit diagonal times 2^-53, from the
+matrix itself."""
 import numpy as np
 import pytest
 
@@ -13,7 +14,7 @@ from oracle import multigrid
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dims", [(1, 3, 3), (4, 4, 2), (2, 2, 2), (3, 3, 5), (1, 2, 1), (6, 1, 2), (12, 5, 4)])
+@pytest.mark.parametrize("dims", [(1, 3, 3), (4, 4, 2), (2, 2, 2), (3, 3, 5), (1, 2, 1), (6, 1, 2), (12, 5, 4), (40, 1, 1)])
 @pytest.mark.parametrize("lo", [1e-3, 0.3])
 def test_direct_solve(dims, lo):
     g, pb, rho, H = make_case(dims, 1, seed=91, lo=lo)
