@@ -505,10 +505,15 @@ __global__ void k_transpose(const double* __restrict__ W, double* __restrict__ W
 // batches of loads (and of the order behind them: 22 us), now of two.
 // FP64 matrices: FP64 sums.  FP32 matrices: every product and sum with its
 // exact rounding error carried in a second FP32 word (TwoProduct by fused
-// multiply-add, Knuth's TwoSum; the sum is as if accumulated in 48 bits
-// before the one rounding of the result): 9 FP32 instructions per entry
-// where two conversions and an FP64 multiply-add take 48 issue cycles of the
-// SM.
+// multiply-add, Knuth's TwoSum): 12 FP32 instructions per entry where two
+// conversions and an FP64 multiply-add take 48 issue cycles of the SM.
+// Against exact sums of the same entries (rows of 1 to 1911, with and without
+// cancellation) the two words are off by at most 2^-46.4 of the sum of the
+// terms' sizes, FP64 sums by 2^-51.2, and both round to the same FP32 number;
+// the entries themselves are rounded to 2^-24.  The second word needs the
+// exponents between: with every term below 2^-80 (its errors would underflow)
+// or one at 2^100 or more (a sum could overflow before it cancels) the row is
+// summed in FP64, unless all its terms are exactly 0 (fixed DOFs).
 __device__ __forceinline__ void two_sum_into(float& s, float& c, float p) {
     const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
     c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b)));
@@ -518,15 +523,17 @@ constexpr int kGemv = 128;
 template <typename T, bool LOWER>
 __global__ void __launch_bounds__(kGemv) k_trigemv(int n, int npad, const T* __restrict__ M, const T* __restrict__ v,
                                                    T* __restrict__ y, const int* __restrict__ order) {
-    __shared__ T red[2][kGemv / 32];
+    __shared__ T red[3][kGemv / 32];
     const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int j1 = LOWER ? row + 1 : n;
     const T* mr = M + (long long)row * npad;
     T s = T(0);
-    [[maybe_unused]] float c = 0.0f;
+    [[maybe_unused]] float c = 0.0f, largest = 0.0f, factor = 0.0f;   // factor: > 0 once a term is not 0
     auto add = [&](T a, T b) {
         if constexpr (std::is_same<T, float>::value) {
             const float p = __fmul_rn(a, b);
+            largest = fmaxf(largest, fabsf(p));
+            factor = fmaxf(factor, fminf(fabsf(a), fabsf(b)));
             c = __fadd_rn(c, __fmaf_rn(a, b, -p));
             two_sum_into(s, c, p);
         } else {
@@ -563,11 +570,30 @@ __global__ void __launch_bounds__(kGemv) k_trigemv(int n, int npad, const T* __r
         if constexpr (std::is_same<T, float>::value) co = __shfl_xor_sync(0xffffffffu, c, o);
         merge(so, co);
     }
+    if constexpr (std::is_same<T, float>::value) {
+        largest = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(largest)));
+        if (largest == 0.0f && !__any_sync(0xffffffffu, factor > 0.0f)) largest = -1.0f;
+    }
     if (lane == 0) {
         red[0][w] = s;
         red[1][w] = (T)c;
+        red[2][w] = (T)largest;
     }
     __syncthreads();
+    if constexpr (std::is_same<T, float>::value) {
+#pragma unroll
+        for (int q = 0; q < kGemv / 32; ++q) largest = fmaxf(largest, red[2][q]);
+        if (largest >= 0.0f && !(largest >= 0x1p-80f && largest < 0x1p100f)) {   // (the same for the whole block)
+            __shared__ double sums[kGemv / 32];
+            double d = 0.0;
+            for (int j = (LOWER ? 0 : row) + tid; j < j1; j += kGemv) d = fma((double)mr[j], (double)v[LOWER ? order[j] : j], d);
+            for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (lane == 0) sums[w] = d;
+            __syncthreads();
+            if (tid == 0) y[LOWER ? row : order[row]] = (float)((sums[0] + sums[1]) + (sums[2] + sums[3]));
+            return;
+        }
+    }
     if (tid == 0) {
 #pragma unroll
         for (int q = 1; q < kGemv / 32; ++q) merge(red[0][q], (float)red[1][q]);
