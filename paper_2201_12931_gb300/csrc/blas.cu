@@ -288,10 +288,11 @@ struct Front {
 //
 // One CTA per chain: a step of two chains takes as long as one of one.
 // L goes back to the block (zeros above the diagonal), L^-1 to Dk (block kb:
-// TB x TB row-major at Dk + kb TB^2).  A non-positive or non-finite pivot sets
-// info to its row + 1 (first one wins) and continues with pivot 1.
-__global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int npad, Front f, int* info,
-                                                    double* __restrict__ Dk) {
+// TB x TB row-major at Dk + kb TB^2).  After a non-positive or non-finite pivot
+// the factorization continues with pivot 1; info ends as n minus the smallest
+// DOF (order: of each row) whose pivot failed, whichever block finds it first.
+__global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int n, int npad, Front f, int* info,
+                                                    const int* __restrict__ order, double* __restrict__ Dk) {
     static_assert(TB == 32, "a lane per row");
     __shared__ double col[TB][TB + 1], ucol[TB][TB + 1];   // pivot columns and U's (rows below the diagonal)
     __shared__ double next[2][TB], piv[TB], root[TB];
@@ -323,7 +324,7 @@ __global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int 
         double d = __shfl_sync(0xffffffffu, v, j);
         const int hi = __double2hiint(d), lo = __double2loint(d);
         if (!((hi > 0 || (hi == 0 && lo != 0)) && hi < 0x7ff00000)) {   // not positive and finite
-            if (lane == 0) atomicCAS(info, 0, (int)(base + j) + 1);
+            if (lane == 0) atomicMax(info, n - (base + j < n ? order[base + j] : n - 1));
             d = 1.0;
         }
         // v / d = v y0 (1 + e + e^2) with e = 1 - d y0: v y0 is off the chain
@@ -700,7 +701,7 @@ void fill(const Ctx& c, long long n, double* v, double value) {
 inline int band_blocks(int band) { return (band + TB - 1) / TB; }
 
 void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A, double* W, int n, int npad, int band,
-                  int* info, double* Dk) {
+                  int* info, const int* order, double* Dk) {
     // The Cholesky factor of a banded matrix keeps its band, so the panel and
     // the trailing update of a step touch only the bb block rows below it; the
     // blocks left out are zero in A and L alike.  Two chains of `a` blocks run
@@ -746,7 +747,7 @@ void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A,
         }
         const int m = std::max(f.m[0], f.m[1]), cols = f.kb[0] - f.c0[0] + 1, nz = f.chains;
         const bool sep = f.m[0] > f.m1[0] || f.m[1] > f.m1[1];
-        k_potrf_diag<<<nz, 512, 0, c.s>>>(A, npad, f, info, Dk);
+        k_potrf_diag<<<nz, 512, 0, c.s>>>(A, n, npad, f, info, order, Dk);
         TOPO_LAUNCH_CHECK(c);
         if (m > 0) {
             k_trsm_panel<<<dim3(TB / kStrip, m, nz), dim3(TB, kStrip), 0, c.s>>>(A, npad, f, Dk);

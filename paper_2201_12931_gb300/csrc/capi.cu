@@ -233,7 +233,7 @@ topo_status ensure_coarse(topo_grid* h) {
                         cs.A, cs.npad, cs.order);
         const bool fork = cc.s == h->cap_stream && h->side_stream && h->side_event;   // capturing
         chol_inverse(cc, fork ? h->side_stream : cc.s, h->side_event, cs.A, cs.W64, cs.n, cs.npad, band, cs.info,
-                     cs.Dk);
+                     cs.order, cs.Dk);
         transpose_dense(cc, cs.W64, cs.WT64, cs.npad);
         const long long n2 = (long long)cs.npad * cs.npad;
         convert<double, float>(cc, n2, cs.W64, cs.W32);
@@ -261,7 +261,7 @@ topo_status ensure_coarse(topo_grid* h) {
     CK(h, cudaMemcpyAsync(&info, cs.info, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     if (info != 0)
-        return fail(h, TOPO_BREAKDOWN, "coarsest-grid matrix not positive definite at row " + std::to_string(info - 1));
+        return fail(h, TOPO_BREAKDOWN, "coarsest-grid matrix not positive definite at row " + std::to_string(cs.n - info));
     h->coarse_dirty = false;
     return TOPO_OK;
 }

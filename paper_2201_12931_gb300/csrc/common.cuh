@@ -89,7 +89,7 @@ struct Coarse {           // dense coarsest-grid solve: K_c^-1 = W^T W, W = L^-1
     float* WT32 = nullptr;
     double* y64 = nullptr;    // temporaries of length npad
     float* y32 = nullptr;
-    int* info = nullptr;      // device: first non-positive pivot + 1 (0 = ok)
+    int* info = nullptr;      // device: n - smallest DOF with a non-positive pivot (0 = ok)
     int* order = nullptr;     // DOF of the level's node order at each row: nodes along the shortest axis first, then two-ended
     double* Dk = nullptr;     // inverses of the 32 x 32 diagonal blocks of L (npad x 32)
 };
@@ -355,13 +355,14 @@ void fill(const Ctx& c, long long n, double* v, double value);
 // dense coarse solve
 // A = L L^T in place and W = L^-1 for n rows in two-ended order (see
 // coarse_chain).  band: half-bandwidth of A in entries before the reordering
-// (npad for a dense matrix); Dk (npad x 32 doubles) receives the inverses of the
-// 32 x 32 diagonal blocks of L.  The inverse of a block row needs the factor
+// (npad for a dense matrix); order: the DOF of each row; Dk (npad x 32 doubles)
+// receives the inverses of the 32 x 32 diagonal blocks of L; info: n minus the
+// smallest DOF whose pivot is not positive, 0 if there is none.  The inverse of a block row needs the factor
 // up to its block column only: with side != c.s (stream capture) its launches
 // go to that stream, ordered by the event, beside the chain of diagonal
 // blocks, and are joined at the end.
 void chol_inverse(const Ctx& c, cudaStream_t side, cudaEvent_t ready, double* A, double* W, int n, int npad, int band,
-                  int* info, double* Dk);
+                  int* info, const int* order, double* Dk);
 void transpose_dense(const Ctx& c, const double* W, double* WT, int npad);
 template <typename T>
 void coarse_apply(const Ctx& c, const Coarse& cs, const T* W, const T* WT, const T* rhs, T* y, T* out);
