@@ -108,7 +108,9 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     T st00[3] = {}, st10[3] = {}, st01[3] = {}, st11[3] = {};
     T stE = T(0);
     double dot = 0.0;
+    constexpr bool kDotF = DOT && (kDF || std::is_same<T, float>::value);
     [[maybe_unused]] float dotf = 0.0f;
+    [[maybe_unused]] dfl dotp(0.0f, 0.0f);
     // per-plane register slots, slot = (plane - first) & 3: own node raw u, f, mask,
     // the column modulus of the layer below the plane, and (two slots) the
     // halo node; planes P-2 .. P+1 are live in step P, so no copies occur.
@@ -358,9 +360,10 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
                 stv(o + c, r[c]);
             }
             if constexpr (DOT) {
-                // FP32 kernels: FP32 per thread (one column of a z chunk),
-                // FP64 across threads and CTAs, fixed order
-                if constexpr (kDF || std::is_same<T, float>::value) dotf += d32;
+                // FP32 kernels: FP32 over at most eight planes of a thread's
+                // column, a pair of FP32 words over the column, FP64 beyond,
+                // fixed order
+                if constexpr (kDotF) dotf += d32;
                 else dot += (double)d32;
             }
         }
@@ -430,6 +433,14 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     const int Pfirst = kz0 - 1;
     fetch(S0{}, Pfirst);
     for (int P = Pfirst; P <= kz1 + 1; P += NS) {
+        // the rounding of a dot product must not depend on how long a chunk the
+        // launch geometry takes: the FP32 sum moves on every eight planes (into
+        // an FP64 sum, on the slow pipe, 768x384x384 steps took 0.4 % longer)
+        if constexpr (kDotF)
+            if (((P - Pfirst) & 7) == 0) {
+                dotp += dfl(dotf, 0.0f);
+                dotf = 0.0f;
+            }
         step(S0{}, P);
         step(S1{}, P + 1);
         if constexpr (NS == 4) {
@@ -439,7 +450,8 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
         }
     }
     if (DOT) {
-        double v = (kDF || std::is_same<T, float>::value) ? (double)dotf : dot;
+        if constexpr (kDotF) dotp += dfl(dotf, 0.0f);
+        double v = kDotF ? widen(dotp.h) + widen(dotp.l) : dot;   // (one FP64 instruction)
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         const int w = tid >> 5, l = tid & 31;
         if (l == 0) sred[w] = v;
