@@ -128,9 +128,6 @@ topo_status alloc_precision(topo_grid* h, bool fp64) {
         ALLOC(h, h->p, n0);
         ALLOC(h, h->q, n0);
         for (auto& d : h->dring64) ALLOC(h, d, n0);
-        size_t el = 0;
-        for (auto& lv : h->lev) el = std::max(el, lv.p64.scratch());
-        if (el > 0) ALLOC(h, h->el64, el);
         h->fp64_ready = true;
     } else {
         ALLOC(h, h->r32, n0);
@@ -141,6 +138,15 @@ topo_status alloc_precision(topo_grid* h, bool fp64) {
         for (auto& d : h->dring32) ALLOC(h, d, n0);
         h->fp32_ready = true;
     }
+    return TOPO_OK;
+}
+
+// scratch of the FP64 operators by elements: FP64 handles, and others once they
+// run an FP64 operator or V-cycle
+topo_status ensure_el64(topo_grid* h) {
+    size_t el = 0;
+    for (auto& lv : h->lev) el = std::max(el, lv.p64.scratch());
+    if (el > 0 && !h->el64) ALLOC(h, h->el64, el);
     return TOPO_OK;
 }
 
@@ -494,6 +500,7 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
     h->cs.n = (int)std::min<long long>(3 * h->lev[h->L - 1].g.nn, 1LL << 30);
     h->cs.npad = (h->cs.n + 31) / 32 * 32;
     TRY(alloc_precision(h, p.precision == TOPO_FP64));
+    if (p.precision == TOPO_FP64) TRY(ensure_el64(h));
     if (p.precision == TOPO_MIXED_BF16) TRY(alloc_bf16(h));
     if (cudaMallocHost((void**)&h->host_sc, sizeof(Scalars)) != cudaSuccess) {
         h->host_sc = nullptr;
@@ -936,6 +943,8 @@ static topo_status level_op(topo_grid* h, int level, int precision, int op, cons
         if (stencil_df(c, mode, lv.op64, *h->mkdf, lv.E64, lv.mask, u, f, out, nullptr, nullptr) < 0)
             return fail(h, TOPO_BADARG, "double-FP32 kernel: mode not available");
     } else if (precision == TOPO_FP64) {
+        s = ensure_el64(h);
+        if (s != TOPO_OK) return s;
         if (op == OP_JACOBI) ensure_dinv64(h);
         op_apply<double>(h, mode, level, u, f, out, nullptr);
     } else {
@@ -997,6 +1006,8 @@ topo_status topo_vcycle(topo_handle h, int precision, const double* r_dev, doubl
     Level& l0 = h->lev[0];
     const long long n = 3 * l0.g.nn;
     if (precision == TOPO_FP64) {
+        s = ensure_el64(h);
+        if (s != TOPO_OK) return s;
         ensure_dinv64(h);
         vcycle<double>(h, 0, r_dev, z_dev, l0.v64.a, nullptr);
     } else if (precision == TOPO_MIXED_BF16) {
