@@ -32,6 +32,12 @@
  *     message of the last failure is available from topo_last_error.  After
  *     TOPO_CUDA the handle may be unusable and should be destroyed.
  *   - a handle is not thread-safe: one host thread at a time per handle.
+ *   - stream capture: calls that neither return host values nor allocate can
+ *     be captured (run each once before).  A filter radius other than the
+ *     last one used is TOPO_BADARG while the stream is being captured: its
+ *     weights are computed once and kept (a captured filter call is replayed
+ *     while its radius is still the last one used).  A captured FP64 sweep or V-cycle
+ *     forms the Jacobi diagonals of the density at the time of the replay.
  */
 #ifndef TOPO_GB300_H
 #define TOPO_GB300_H

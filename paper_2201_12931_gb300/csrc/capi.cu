@@ -272,9 +272,21 @@ topo_status ensure_coarse(topo_grid* h) {
     return TOPO_OK;
 }
 
+// whether launches on the handle's stream are only recorded
+bool capturing(topo_grid* h) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+        cudaGetLastError();   // (the legacy stream while another one is captured)
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 topo_status prepare_filter(topo_grid* h, double r) {
     if (!(r > 0.0) || r > 6.0) return fail(h, TOPO_BADARG, "filter radius must be in (0, 6]");
     if (r == h->S_radius) return TOPO_OK;
+    // (the weights are kept for later calls: they have to be computed, not recorded)
+    if (capturing(h)) return fail(h, TOPO_BADARG, "filter weights of a new radius cannot be formed during stream capture");
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
     filter_plan(g, r, h->nsm, &h->filt);
@@ -287,6 +299,7 @@ topo_status prepare_filter(topo_grid* h, double r) {
 // radius prepared last
 topo_status prepare_dv(topo_grid* h) {
     if (h->dv_radius == h->S_radius) return TOPO_OK;
+    if (capturing(h)) return fail(h, TOPO_BADARG, "the OC update cannot be captured");
     if (!h->rdv_cache) ALLOC(h, h->rdv_cache, h->lev[0].g.ne);
     filter_launch(h->ctx(), h->lev[0].g, h->filt, 1, nullptr, nullptr, 0.0, h->stab, h->dv_cache);
     reciprocal(h->ctx(), h->lev[0].g.ne, h->dv_cache, h->rdv_cache);
@@ -340,14 +353,17 @@ topo_status check_handle(topo_grid* h) {
 
 }  // namespace
 
+// In a captured stream the diagonals are formed in the graph itself, at every
+// replay: the density may be another one by then
 void topo::ensure_dinv64(topo_grid* h) {
-    if (!h->dinv64_dirty) return;
+    const bool recorded = capturing(h);
+    if (!h->dinv64_dirty && !recorded) return;
     const Ctx c = h->ctx();
     for (int l = 0; l < h->L; ++l) {
         Level& lv = h->lev[l];
         diag_inverse<double>(c, lv.g, lv.E64, h->mk64->kdiag, lv.Dinv64);
     }
-    h->dinv64_dirty = false;
+    if (!recorded) h->dinv64_dirty = false;
 }
 
 void topo::set_global_error(const std::string& msg) { g_create_err = msg; }
