@@ -471,12 +471,13 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
         lv.scale = (double)(1 << l);
         lv.op32 = op_launch32(lv.g, nsm);
         lv.op64 = op_launch64(lv.g, nsm);
+        lv.opdf = op_launch_df(lv.g, nsm);
         lv.optc = op_launch_tc(lv.g, nsm);
         lv.brick = lv.g.nn <= kBrickMax;
         if (lv.brick) h->npartials = std::max(h->npartials, brick_ctas(lv.g));
         if (lv.g.ne <= kOp64Max) lv.p64 = op64_plan(lv.g, nsm);
         h->npartials = std::max(h->npartials, (long long)lv.p64.blocks);
-        h->npartials = std::max(h->npartials, std::max(lv.op32.ctas(), std::max(lv.op64.ctas(), lv.optc.ctas())));
+        for (const OpLaunch* L : {&lv.op32, &lv.op64, &lv.opdf, &lv.optc}) h->npartials = std::max(h->npartials, L->ctas());
     }
     topo_status st;
 #define TRY(expr)                          \
@@ -956,7 +957,7 @@ static topo_status level_op(topo_grid* h, int level, int precision, int op, cons
     } else if (precision == TOPO_DF32) {
         if (h->prm.homogenize == 2 && level > 0)
             return fail(h, TOPO_BADARG, "double-FP32 kernel: not for stored Galerkin levels");
-        if (stencil_df(c, mode, lv.op64, *h->mkdf, lv.E64, lv.mask, u, f, out, nullptr, nullptr) < 0)
+        if (stencil_df(c, mode, lv.opdf, *h->mkdf, lv.E64, lv.mask, u, f, out, nullptr, nullptr) < 0)
             return fail(h, TOPO_BADARG, "double-FP32 kernel: mode not available");
     } else if (precision == TOPO_FP64) {
         s = ensure_el64(h);

@@ -65,7 +65,7 @@ struct Level {
     bf16* hb = nullptr;
     double* Ke64 = nullptr;   // stored Galerkin element matrices (homogenize = 2, levels >= 1)
     float* Ke32 = nullptr;
-    OpLaunch op32, op64;      // operator launch geometry per precision
+    OpLaunch op32, op64, opdf;   // operator launch geometry per precision
     OpLaunch optc;            // tensor-core FP32 operator (tc_op.cu)
     Op64Plan p64;             // FP64 operator by elements (op64.cu)
     bool brick = false;       // FP32 operators by bricks (op_brick.cu)
@@ -216,6 +216,7 @@ enum StencilMode { ST_APPLY = 0, ST_JACOBI = 1, ST_RESID = 2, ST_JACOBI0 = 3, ST
 // nsm: multiprocessors of the device (wave-aware z chunking)
 OpLaunch op_launch32(const Geom& g, int nsm);
 OpLaunch op_launch64(const Geom& g, int nsm);
+OpLaunch op_launch_df(const Geom& g, int nsm);
 template <typename T>
 int stencil(const Ctx& c, int mode, const OpLaunch& L, const ModalK<T>& mk, const T* E, const uint8_t* mask,
             const T* u, const T* f, T* out, T omega, double* dot_partials, const T* Dinv, T* pout = nullptr,
@@ -257,7 +258,7 @@ int brick_apply(const Ctx& c, int mode, const Geom& g, const ModalK<float>& mk, 
 void brick_restrict(const Ctx& c, const Geom& g, const ModalK<float>& mk, const float* E, const uint8_t* mask,
                     const float* u, const float* f, const uint8_t* maskc, float* fc);
 // ---- tc_op.cu: FP32 operators with the element products on tcgen05 tensor cores
-OpLaunch op_launch(const Geom& g, int ty, int resident_ctas);
+OpLaunch op_launch(const Geom& g, int ty, int resident_ctas, bool fp64 = false);
 OpLaunch op_launch_tc(const Geom& g, int nsm);
 constexpr int kTcBWords = 2304;
 // host: shared-memory image of B = [K0_hi | K0_lo | K0_hi] (TF32), kTcBWords words

@@ -473,7 +473,7 @@ static double residual_df(topo_grid* h) {
         }
         cudaEventRecord(h->prof_ev[2 * h->prof_n], h->stream);
     }
-    const int np = stencil_df(c, ST_RESID, l0.op64, *h->mkdf, l0.E64, l0.mask, h->x, h->f, nullptr, h->r32,
+    const int np = stencil_df(c, ST_RESID, l0.opdf, *h->mkdf, l0.E64, l0.mask, h->x, h->f, nullptr, h->r32,
                               h->partials);
     if (rec) {
         cudaEventRecord(h->prof_ev[2 * h->prof_n + 1], h->stream);

@@ -682,7 +682,29 @@ __global__ void __launch_bounds__(256) k_energy_sens_z(ModalCoef mc, const doubl
 // groups of four steps: V-cycle over 128x64x64 elements 212 -> 196 -> 193 us,
 // operators of 256x128x128 elements 561 -> 558 -> 543 us, double-FP32 operators
 // of 151x77x93 elements 322 -> 296 us.
-OpLaunch op_launch(const Geom& g, int ty, int resident_ctas) {
+// fp64: the FP64 pipe bounds a CTA, one to an SM, so a chunk costs the cz + 1
+// layers that it computes and about one more for the rest, and the chunks
+// are dealt out as SMs become free (fp64_layers: 9.9 to 10.8 us a layer over
+// grids of 3456 to 4 million elements).  K.u over 160x96x80 elements with the
+// FP32 rule: 621 us (252 CTAs of 29 layers, in two waves), with this one 564
+// (756 of 11, in five); over 256x128x128 1814 and 1730 us.
+static double fp64_layers(long long xy, int cz, int NZ, int sms) {
+    const int chunks = (NZ + cz - 1) / cz;
+    const long long full = xy * (chunks - 1), rem = full % sms;
+    const double c1 = cz + 2.0, c2 = NZ - (chunks - 1) * cz + 2.0;   // the last chunk of a column is shorter
+    // the full chunks leave rem SMs busy a chunk longer than the others
+    double early = (double)(full / sms) * c1, late = early + c1, end = rem > 0 ? late : early;
+    for (long long left = xy; left > 0;) {
+        const bool first = rem == 0 || early <= late;
+        left -= first ? sms - rem : rem;
+        double& t = first ? early : late;
+        t += c2;
+        end = std::max(end, t);
+    }
+    return end;
+}
+
+OpLaunch op_launch(const Geom& g, int ty, int resident_ctas, bool fp64) {
     OpLaunch L;
     L.g = g;
     L.gx = (g.nx + 1 + kOpTX - 2) / (kOpTX - 1);
@@ -694,7 +716,7 @@ OpLaunch op_launch(const Geom& g, int ty, int resident_ctas) {
         const int cz = std::max((NZ + gz - 1) / gz, std::min(4, NZ));   // at least 4 planes
         const long long chunks = (NZ + cz - 1) / cz;
         const long long waves = (xy * chunks + resident_ctas - 1) / resident_ctas;
-        const double cost = (double)waves * ((cz + 4) / 2 * 2 + 1.5);
+        const double cost = fp64 ? fp64_layers(xy, cz, NZ, resident_ctas) : (double)waves * ((cz + 4) / 2 * 2 + 1.5);
         if (best < 0.0 || cost < best) {
             best = cost;
             L.cz = cz;
@@ -705,9 +727,10 @@ OpLaunch op_launch(const Geom& g, int ty, int resident_ctas) {
     return L;
 }
 
-// resident CTAs per SM: 2 for the FP32 kernel (launch bounds 256 x 2), 1 for FP64
+// resident CTAs per SM: 2 for the FP32 kernel (launch bounds 256 x 2), 1 for FP64 and double-FP32
 OpLaunch op_launch32(const Geom& g, int nsm) { return op_launch(g, op_ty<float>(), 2 * nsm); }
-OpLaunch op_launch64(const Geom& g, int nsm) { return op_launch(g, op_ty<double>(), nsm); }
+OpLaunch op_launch64(const Geom& g, int nsm) { return op_launch(g, op_ty<double>(), nsm, true); }
+OpLaunch op_launch_df(const Geom& g, int nsm) { return op_launch(g, op_ty<dfl>(), nsm); }
 
 template <typename T>
 int stencil(const Ctx& c, int mode, const OpLaunch& L, const ModalK<T>& mk, const T* E, const uint8_t* mask,
