@@ -240,11 +240,6 @@ __global__ void __launch_bounds__(256) k_convert(long long n, const S* __restric
     for (; i < n; i += stride) d[i] = conv(s[i]);
 }
 
-__global__ void k_fill(long long n, double* __restrict__ v, double value) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        v[i] = value;
-}
-
 __global__ void k_axpy_f32(long long n, const float* __restrict__ d, double* __restrict__ x) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         x[i] += (double)d[i];
@@ -690,11 +685,6 @@ void zero(const Ctx& c, long long n, T* v) {
 }
 template void zero<double>(const Ctx&, long long, double*);
 template void zero<float>(const Ctx&, long long, float*);
-
-void fill(const Ctx& c, long long n, double* v, double value) {
-    k_fill<<<grid_for(n, 256) > 8192 ? 8192 : grid_for(n, 256), 256, 0, c.s>>>(n, v, value);
-    TOPO_LAUNCH_CHECK(c);
-}
 
 // Blocks of a banded matrix (A_ij = 0 for |i - j| > band) that can be nonzero
 // below the diagonal block of block column kb: block rows kb+1 .. kb+bb.

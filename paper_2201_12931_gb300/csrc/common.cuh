@@ -360,7 +360,6 @@ void convert(const Ctx& c, long long n, const S* src, D* dst);
 void axpy_f32_into_f64(const Ctx& c, long long n, const float* d, double* x);
 template <typename T>
 void zero(const Ctx& c, long long n, T* v);
-void fill(const Ctx& c, long long n, double* v, double value);
 // dense coarse solve
 // A = L L^T in place and W = L^-1 for n rows in two-ended order (see
 // coarse_chain).  band: half-bandwidth of A in entries before the reordering

@@ -83,8 +83,6 @@ __host__ __device__ __forceinline__ dfl df_from_double(double x) {
 
 __host__ __device__ __forceinline__ dfl::dfl(double x) : dfl(df_from_double(x)) {}
 
-__host__ __device__ __forceinline__ double df_to_double(dfl a) { return (double)a.h + (double)a.l; }
-
 #ifdef __CUDACC__
 __device__ __forceinline__ float df_to_float(dfl a) { return __fadd_rn(a.h, a.l); }
 

@@ -220,14 +220,8 @@ int op64_apply(const Ctx& c, int mode, const Geom& g, const Op64Plan& p, const M
     else EL(IN_U);
     TOPO_LAUNCH_CHECK(c);
     switch (mode) {
-        case ST_APPLY:
-            if (dot) ND(ST_APPLY, true);
-            else ND(ST_APPLY, false);
-            break;
-        case ST_APPLY_P:
-            if (dot) ND(ST_APPLY_P, true);
-            else ND(ST_APPLY_P, false);
-            break;
+        case ST_APPLY: ND(ST_APPLY, false); break;
+        case ST_APPLY_P: ND(ST_APPLY_P, true); break;   // CG only: always with p.q
         case ST_JACOBI:
             if (dot) ND(ST_JACOBI, true);
             else ND(ST_JACOBI, false);
@@ -241,7 +235,7 @@ int op64_apply(const Ctx& c, int mode, const Geom& g, const Op64Plan& p, const M
     TOPO_LAUNCH_CHECK(c);
 #undef EL
 #undef ND
-    return mode == ST_JACOBI2 || !dot ? 0 : (tail.kind != TAIL_NONE ? -1 : p.blocks);
+    return mode == ST_JACOBI2 || mode == ST_APPLY || !dot ? 0 : (tail.kind != TAIL_NONE ? -1 : p.blocks);
 }
 
 }  // namespace topo

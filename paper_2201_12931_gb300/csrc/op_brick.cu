@@ -321,15 +321,12 @@ cudaError_t brick_init() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_brick_restrict, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem);
     set(k_brick<ST_APPLY_P, true, false>);
-    set(k_brick<ST_APPLY_P, false, false>);
-    set(k_brick<ST_APPLY, true, false>);
     set(k_brick<ST_APPLY, false, false>);
     set(k_brick<ST_JACOBI, true, true>);
     set(k_brick<ST_JACOBI, false, true>);
     set(k_brick<ST_JACOBI, true, false>);
     set(k_brick<ST_JACOBI, false, false>);
     set(k_brick<ST_JACOBI2, false, false>);
-    set(k_brick<ST_RESID, true, false>);
     set(k_brick<ST_RESID, false, false>);
     return e;
 }
@@ -345,14 +342,8 @@ int brick_apply(const Ctx& c, int mode, const Geom& g, const ModalK<float>& mk, 
     const Coarser cr{ec, maskc};
 #define GO(MODE, DOT, PRO) launch<MODE, DOT, PRO>(c, g, mk, E, mask, u, f, out, omega, dot, Dinv, pout, beta, cr, tail)
     switch (mode) {
-        case ST_APPLY_P:
-            if (dot) GO(ST_APPLY_P, true, false);
-            else GO(ST_APPLY_P, false, false);
-            break;
-        case ST_APPLY:
-            if (dot) GO(ST_APPLY, true, false);
-            else GO(ST_APPLY, false, false);
-            break;
+        case ST_APPLY_P: GO(ST_APPLY_P, true, false); break;   // CG only: always with p.q
+        case ST_APPLY: GO(ST_APPLY, false, false); return 0;
         case ST_JACOBI:
             if (ec && dot) GO(ST_JACOBI, true, true);
             else if (ec) GO(ST_JACOBI, false, true);
@@ -360,10 +351,7 @@ int brick_apply(const Ctx& c, int mode, const Geom& g, const ModalK<float>& mk, 
             else GO(ST_JACOBI, false, false);
             break;
         case ST_JACOBI2: GO(ST_JACOBI2, false, false); return 0;
-        default:
-            if (dot) GO(ST_RESID, true, false);
-            else GO(ST_RESID, false, false);
-            break;
+        default: GO(ST_RESID, false, false); return 0;
     }
 #undef GO
     return dot ? (tail.kind != TAIL_NONE ? -1 : (int)brick_ctas(g)) : 0;

@@ -88,7 +88,6 @@ __global__ void __launch_bounds__(kOpTX * op_ty<T>(), sizeof(T) == 4 ? 2 : 1)
     const int hsx = tid < TY + 1 ? TX : tid - TY - 1;
     const int hsy = tid < TY + 1 ? tid : TY;
     const int hx = i0 - 1 + hsx, hy = j0 - 1 + hsy;
-    const bool halo_ok = has_halo && hx >= 0 && hx < NX && hy >= 0 && hy < NY;
     // 32-bit vector indices (topo_create_grid keeps 3 * nodes below 2^31):
     // fewer address instructions and registers
     using Ix = int;
