@@ -308,7 +308,10 @@ topo_status topo_level_density(topo_handle h, int level, double* rho_dev_out);
  * TOPO_MIXED (FP32 vectors and arithmetic) or TOPO_MIXED_BF16 (FP32
  * arithmetic, FP32 right-hand sides and residuals, smoother iterates and
  * prolongated corrections stored in BF16 on every level above the coarsest;
- * the level-0 result is FP32).  r and z: device FP64, 3*nodes each. */
+ * the level-0 result is FP32).  The FP32 coarsest solve multiplies FP32
+ * matrices and vectors and adds in pairs of FP32 words (2^-46 of the terms'
+ * sizes; FP64 sums for rows whose terms are all below 2^-80 or reach 2^100)
+ * before it rounds to FP32.  r and z: device FP64, 3*nodes each. */
 topo_status topo_vcycle(topo_handle h, int precision, const double* r_dev, double* z_dev);
 
 /* Statistics of the last topo_solve_state. */

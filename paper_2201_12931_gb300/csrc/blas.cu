@@ -3,8 +3,10 @@
 // solve on the coarsest grid (Algorithm 3 "Solve the problem directly"):
 // blocked right-looking Cholesky K_c = L L^T, explicit W = L^-1, and per
 // application u = W^T (W r) as two triangular matrix-vector products.
-// Reductions use a fixed grid of kRedBlocks blocks and a fixed-order second
-// pass, so results are bitwise reproducible run to run.
+// Reductions add their blocks' partial sums in a fixed order, in a second pass
+// (k_reduce_to, k_cg_scalar) or in the last block to finish (tail.cuh), over
+// grids that are fixed per handle, so results are bitwise
+// reproducible run to run.
 #include <math.h>
 
 #include <algorithm>
