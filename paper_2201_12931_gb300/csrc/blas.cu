@@ -317,11 +317,12 @@ __global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int 
         v = A[(base + lane) * npad + base];
         if (lane >= 1) vn = A[(base + lane) * npad + base + 1];
     }
+    unsigned failed = 0u;                // warp 0: rows whose pivot is not positive and finite
     auto publish = [&](int j) {   // warp 0: v is column j, up to date
         double d = __shfl_sync(0xffffffffu, v, j);
         const int hi = __double2hiint(d), lo = __double2loint(d);
         if (!((hi > 0 || (hi == 0 && lo != 0)) && hi < 0x7ff00000)) {   // not positive and finite
-            if (lane == 0) atomicMax(info, n - (base + j < n ? order[base + j] : n - 1));
+            failed |= 1u << j;
             d = 1.0;
         }
         // v / d = v y0 (1 + e + e^2) with e = 1 - d y0: v y0 is off the chain
@@ -376,7 +377,11 @@ __global__ void __launch_bounds__(512) k_potrf_diag(double* __restrict__ A, int 
         }
     }
     __syncthreads();
-    if (w == 0) root[lane] = rsqrt(piv[lane]);
+    if (w == 0) {
+        root[lane] = rsqrt(piv[lane]);
+        // (noted after the chain of pivots: an order lookup in it took 1 us a block)
+        if ((failed >> lane) & 1u) atomicMax(info, n - (base + lane < n ? order[base + lane] : n - 1));
+    }
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
