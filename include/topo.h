@@ -196,7 +196,7 @@ topo_status topo_state_step_host(topo_handle h, const double* rho_host, double r
  *   transpose = 0: out_e = sum_i w_ei in_i / S_e
  *   transpose = 1: out_i = sum_e w_ei in_e / S_e
  * in_dev, out_dev: device, nx*ny*nz FP64, must not overlap.  0 < r <= 6
- * (at most 905 neighbour offsets, summed by symmetry class). */
+ * (at most 905 neighbour offsets, summed by symmetry class or one by one). */
 topo_status topo_filter(topo_handle h, double r, const double* in_dev, double* out_dev,
                         int transpose);
 
@@ -366,10 +366,10 @@ topo_status topo_measure_peak(int kind, void* stream, double* tflops_out, double
  * without a handle: a framework whose caching allocator owns the device
  * memory, or a loop that must not stall on the device-wide synchronisation
  * of cudaMalloc/cudaFree, can call it at any point.  It calls no
- * cudaMalloc, cudaFree or other allocating routine; its scratch (a table
- * of weight sums) lives in one statically sized array of 21 KiB that every
- * GPU loading this library holds until the process exits.  The first call on a device looks up that array's address (make it
- * before any stream capture).  Grids of at most 1,048,576 elements
+ * cudaMalloc, cudaFree or other allocating routine; its scratch (tables
+ * of weight sums) lives in one statically sized array of 42 KiB that every
+ * GPU loading this library holds until the process exits.  The first call on a
+ * device looks up that array's address (make it before any stream capture).  Grids of at most 1,048,576 elements
  * (nx*ny*nz) and radii 0 < r <= 6; larger grids return TOPO_BADARG with a
  * message from topo_last_error(NULL).  in_dev/out_dev: device, nx*ny*nz FP64,
  * must not overlap; stream: cudaStream_t (NULL = legacy default stream).

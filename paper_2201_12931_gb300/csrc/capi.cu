@@ -289,7 +289,7 @@ topo_status prepare_filter(topo_grid* h, double r) {
     if (capturing(h)) return fail(h, TOPO_BADARG, "filter weights of a new radius cannot be formed during stream capture");
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
-    filter_plan(g, r, h->nsm, &h->filt);
+    filter_plan(g, r, h->nsm, true, &h->filt);
     filter_weights(c, g, h->filt, h->stab);
     h->S_radius = r;
     return TOPO_OK;
@@ -301,7 +301,7 @@ topo_status prepare_dv(topo_grid* h) {
     if (h->dv_radius == h->S_radius) return TOPO_OK;
     if (capturing(h)) return fail(h, TOPO_BADARG, "the OC update cannot be captured");
     if (!h->rdv_cache) ALLOC(h, h->rdv_cache, h->lev[0].g.ne);
-    filter_launch(h->ctx(), h->lev[0].g, h->filt, 1, nullptr, nullptr, 0.0, h->stab, h->dv_cache);
+    filter_launch(h->ctx(), h->lev[0].g, h->filt, 1, nullptr, nullptr, 0.0, h->stab, nullptr, h->dv_cache);
     reciprocal(h->ctx(), h->lev[0].g.ne, h->dv_cache, h->rdv_cache);
     h->dv_radius = h->S_radius;
     return TOPO_OK;
@@ -503,7 +503,7 @@ topo_status topo_create_grid(int nx, int ny, int nz, const topo_params* prm, voi
     TRY(dalloc(h, &h->dc_work, g0.ne));
     TRY(dalloc(h, &h->xnew_work, g0.ne));
     TRY(dalloc(h, &h->oc_hi, g0.ne));
-    TRY(dalloc(h, &h->stab, 2 * kFilterTab));
+    TRY(dalloc(h, &h->stab, kFilterTables));
     TRY(dalloc(h, &h->dv_cache, g0.ne));
     TRY(dalloc(h, &h->lam, 8));
     TRY(dalloc(h, &h->dtmp, 8));
@@ -764,7 +764,7 @@ topo_status topo_filter(topo_handle h, double r, const double* in_dev, double* o
     if (s != TOPO_OK) return s;
     const Ctx c = h->ctx();
     const Geom& g = h->lev[0].g;
-    filter_launch(c, g, h->filt, transpose ? 1 : 0, in_dev, nullptr, 0.0, h->stab, out_dev);
+    filter_launch(c, g, h->filt, transpose ? 1 : 0, in_dev, nullptr, 0.0, h->stab, h->xnew_work, out_dev);
     CK(h, cudaGetLastError());
     return TOPO_OK;
 }
@@ -832,7 +832,7 @@ topo_status topo_oc_update(topo_handle h, double r, double move, double volfrac,
     const Geom& g = h->lev[0].g;
     s = prepare_dv(h);
     if (s != TOPO_OK) return s;
-    filter_launch(c, g, h->filt, 1, dc_dev, nullptr, 0.0, h->stab, h->dc_work);
+    filter_launch(c, g, h->filt, 1, dc_dev, nullptr, 0.0, h->stab, h->xnew_work, h->dc_work);
     // q over dc_work, lower bounds in xnew_work, upper bounds in oc_hi
     oc_prepare(c, g.ne, rho_dev_inout, h->dc_work, h->dc_work, h->dv_cache, h->rdv_cache, nullptr, move, h->xnew_work, h->oc_hi,
                h->r, h->oc_ws);
@@ -891,7 +891,7 @@ topo_status topo_sensitivity_filter(topo_handle h, double r, double gamma, const
     if (!(gamma > 0.0)) return fail(h, TOPO_BADARG, "gamma must be positive");
     s = prepare_filter(h, r);
     if (s != TOPO_OK) return s;
-    filter_launch(h->ctx(), h->lev[0].g, h->filt, 2, dc_dev, rho_dev, gamma, h->stab, out_dev);
+    filter_launch(h->ctx(), h->lev[0].g, h->filt, 2, dc_dev, rho_dev, gamma, h->stab, h->xnew_work, out_dev);
     CK(h, cudaGetLastError());
     return TOPO_OK;
 }

@@ -108,12 +108,15 @@ struct PcgGraph {             // a captured launch sequence (a PCG iteration, or
 struct FilterW {
     double w[6][21];
     unsigned bits[21];
+    signed char reach[6][6];      // [c][b]: the largest a with a positive weight, -1: none
 };
 struct FilterPlan {
     FilterW w;
-    int R = 0, tx = 32, cz = 1;   // largest offset; tile width and planes per CTA
+    int R = 0, tx = 32, cz = 1;   // largest offset; tile width and planes per CTA of the march
+    bool near[3] = {};            // by mode: neighbour by neighbour instead of the march
 };
-constexpr int kFilterTab = 11 * 11 * 11;   // weight sums S by distance to the faces; then 1 / S
+// weight sums S by distance to the faces, 1 / S; the same for k_filter_near
+constexpr int kFilterTab = 11 * 11 * 11, kFilterTables = 4 * kFilterTab;
 
 struct Scalars {              // device-resident CG scalars
     double rz, rz_new, pq, rr, alpha, beta, ff, aux;
@@ -156,7 +159,7 @@ struct topo_grid {
     double* G64 = nullptr;          // Galerkin child matrices P_o^T K0 P_o (homogenize = 2)
     double* oc_dv = nullptr;        // active-element indicator of a passive OC step (lazy)
     topo::FilterPlan filt{};        // weights and launch geometry of the filter for S_radius
-    double* stab = nullptr;         // its table of weight sums (2 kFilterTab)
+    double* stab = nullptr;         // its tables of weight sums (kFilterTables)
     double* dv_cache = nullptr;     // H^T 1 for dv_radius
     double* rdv_cache = nullptr;    // its reciprocal (on first use)
     double S_radius = -1.0, dv_radius = -1.0;
@@ -378,14 +381,16 @@ void coarse_apply(const Ctx& c, const Coarse& cs, const T* W, const T* WT, const
 // message returned by topo_last_error(NULL)
 void set_global_error(const std::string& msg);
 // ---- filter.cu -----------------------------------------------------------
-// weights and launch geometry for radius r (0 < r <= 6)
-void filter_plan(const Geom& g, double r, int nsm, FilterPlan* p);
-// fills stab (2 kFilterTab doubles) with the weight sums of the plan's radius
+// weights and launch geometry for radius r (0 < r <= 6); scratch: whether
+// filter_launch gets it
+void filter_plan(const Geom& g, double r, int nsm, bool scratch, FilterPlan* p);
+// fills stab (kFilterTables doubles) with the weight sums of the plan's radius
 void filter_weights(const Ctx& c, const Geom& g, const FilterPlan& p, double* stab);
 // mode 0: out = H in; 1: out = H^T in (in null: H^T 1); 2: the sensitivity
-// filter out = H(rho in) / max(gamma, rho)
+// filter out = H(rho in) / max(gamma, rho).  scratch: one value per element, or
+// null (the values are then formed where they are read)
 void filter_launch(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, const double* in, const double* rho,
-                   double gamma, const double* stab, double* out);
+                   double gamma, const double* stab, double* scratch, double* out);
 // ---- oc.cu ---------------------------------------------------------------
 // OC update: q = x sqrt(max(-dc~, 1e-30) / dv~) (in place over dc~ allowed),
 // move-limit bounds lo / hi, and FP32 copies of (q, lo, hi, dv) in pack (16 B

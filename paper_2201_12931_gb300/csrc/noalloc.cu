@@ -18,8 +18,8 @@ namespace {
 constexpr long long kNoAllocMaxElems = 1LL << 20;   // largest grid: 1,048,576 elements
 constexpr int kNoAllocMaxDevices = 64;
 
-// the table of weight sums (filter_weights)
-__device__ __align__(256) double g_filter_scratch[2 * kFilterTab];
+// the tables of weight sums (filter_weights)
+__device__ __align__(256) double g_filter_scratch[kFilterTables];
 
 std::mutex g_mu;
 double* g_scratch_ptr[kNoAllocMaxDevices] = {};
@@ -90,9 +90,10 @@ extern "C" topo_status topo_filter_noalloc(int nx, int ny, int nz, double r, con
     // weight sums is formed on the device, so no host memory is copied and
     // the launches depend on the arguments alone
     FilterPlan plan;
-    filter_plan(g, r, nsm, &plan);
+    filter_plan(g, r, nsm, false, &plan);
+    plan.near[0] = plan.near[1] = plan.near[2] = plan.near[transpose ? 1 : 0];   // one table of weight sums
     filter_weights(c, g, plan, scratch);
-    filter_launch(c, g, plan, transpose ? 1 : 0, in_dev, nullptr, 0.0, scratch, out_dev);
+    filter_launch(c, g, plan, transpose ? 1 : 0, in_dev, nullptr, 0.0, scratch, nullptr, out_dev);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(TOPO_CUDA, std::string("filter launch: ") + cudaGetErrorString(e));
     return TOPO_OK;
