@@ -242,8 +242,8 @@ int stencil_df(const Ctx& c, int mode, const OpLaunch& L, const ModalK<dfl>& mk,
 // Levels of at most this many elements take op64_apply for every mode but
 // JACOBI0.  What sets the line is memory, not time: the scratch takes 12 (cz + 1)
 // / cz values per element, at most 200 MB up to here.  The z-march is the slower
-// side throughout: K.u over 0.46M elements 160 us by elements and 258 by the
-// march, 1.05M 362 / 512, 1.07M 362 / 438, 1.23M 413 / 564, 4.2M 1361 / 1730.
+// side throughout: K.u over 0.46M elements 160 us by elements and 227 by the
+// march, 1.05M 361 / 511, 1.07M 362 / 437, 1.23M 411 / 562, 4.2M 1355 / 1728.
 constexpr long long kOp64Max = 1LL << 20;
 Op64Plan op64_plan(const Geom& g, int nsm);
 // as stencil(); Dinv is read by JACOBI and JACOBI2; scratch: p.scratch() doubles
@@ -253,10 +253,10 @@ int op64_apply(const Ctx& c, int mode, const Geom& g, const Op64Plan& p, const M
 // ---- op_brick.cu: FP32 operators of small levels ---------------------------
 // Levels of at most this many nodes take brick_apply for every mode but JACOBI0.
 // The two sides cross here: 48 CG iterations with bricks / the z-march on the
-// finest level take 5.03 / 5.17 ms at 71k nodes, 5.46 / 5.57 at 76k, 6.47 / 6.17
-// at 83k, 4.86 / 4.68 at 88k, 5.37 / 4.76 at 109k, 5.68 / 4.75 at 137k and
-// 6.56 / 5.51 at 204k (grids of several shapes).  A V-cycle alone crosses between
-// 99k and 105k: it has no K.p, whose march gains most from a full GPU.
+// finest level take 5.11 / 5.27 ms at 71k nodes, 5.58 / 5.80 at 76k, 6.72 / 6.51
+// at 83k, 4.84 / 4.72 at 88k, 5.37 / 4.85 at 109k, 5.73 / 4.85 at 137k and
+// 6.55 / 5.58 at 204k (grids of several shapes).  A V-cycle alone crosses between
+// 99k and 109k: it has no K.p, whose march gains most from a full GPU.
 constexpr long long kBrickMax = 80000;
 cudaError_t brick_init();   // per device, before the first launch
 long long brick_ctas(const Geom& g);
