@@ -388,7 +388,7 @@ void filter_plan(const Geom& g, double r, int nsm, bool scratch, FilterPlan* p);
 void filter_weights(const Ctx& c, const Geom& g, const FilterPlan& p, double* stab);
 // mode 0: out = H in; 1: out = H^T in (in null: H^T 1); 2: the sensitivity
 // filter out = H(rho in) / max(gamma, rho).  scratch: one value per element, or
-// null (the values are then formed where they are read)
+// null (not for the sensitivity filter; H^T then divides where it reads)
 void filter_launch(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, const double* in, const double* rho,
                    double gamma, const double* stab, double* scratch, double* out);
 // ---- oc.cu ---------------------------------------------------------------

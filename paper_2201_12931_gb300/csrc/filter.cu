@@ -340,13 +340,12 @@ __global__ void __launch_bounds__(256) k_filter_values(int nx, int ny, int nz, c
     }
 }
 
-// without scratch, for H^T 1 and with no neighbours (R = 0) the values are
-// formed where they are read: one launch
+// without scratch (H^T), for H^T 1 and with no neighbours (R = 0) the values
+// are formed where they are read: one launch
 template <int R>
 void launch_near(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, const double* in, const double* rho,
                  double gamma, const double* stab, double* scratch, double* out) {
     const unsigned grid = (unsigned)((g.ne + 255) / 256);
-    const bool form = R == 0 || !scratch || !in;
 #define NEAR(MODE, FORM, IN) \
     k_filter_near<R, MODE, FORM><<<grid, 256, 0, c.s>>>(p.w, g.nx, g.ny, g.nz, IN, rho, gamma, stab, out)
 #define VALUES(MODE)                                                                                   \
@@ -355,10 +354,11 @@ void launch_near(const Ctx& c, const Geom& g, const FilterPlan& p, int mode, con
     NEAR(MODE, false, scratch)
     if (mode == 0) {
         NEAR(0, false, in);
-    } else if (mode == 1 && form) {
+    } else if constexpr (R == 0) {
+        if (mode == 1) NEAR(1, true, in);
+        else NEAR(2, true, in);
+    } else if (mode == 1 && (!scratch || !in)) {
         NEAR(1, true, in);
-    } else if (mode == 2 && form) {
-        NEAR(2, true, in);
     } else if (mode == 1) {
         VALUES(1);
     } else {
