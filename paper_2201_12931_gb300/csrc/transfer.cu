@@ -26,8 +26,10 @@ inline unsigned grid_for(long long n, int threads) {
 // fine plane is summed once per coarse column.  EARLY: the nine values and
 // masks of a plane are loaded before any is used (a value is not loaded behind
 // its mask): a small level's launch is as long as its chain of loads (33x17x17
-// coarse nodes: 10.9 -> 6.9 us); where the grid fills the GPU the extra
-// registers cost more.
+// coarse nodes: 10.9 -> 6.9 us).  In FP64 that takes registers, which cost more
+// once SMs hold more than two CTAs: restriction of 30x30x30 elements
+// 12.1 -> 10.3 us and of 56x56x56 12.4 -> 10.4, but 88x88x88 (540 CTAs) 30.8 ->
+// 37.4, 8x8x1000 (501) 18.5 -> 24.3 and 4000x8x8 (315) 12.5 -> 14.4.
 template <typename T, bool EARLY>
 __global__ void __launch_bounds__(256) k_restrict_z(const uint8_t* __restrict__ maskf, const uint8_t* __restrict__ maskc,
                                                     const T* __restrict__ rf, T* __restrict__ rc, int nxf, int nyf,
@@ -290,7 +292,8 @@ void restrict_residual(const Ctx& c, const Geom& gf, const uint8_t* maskf, const
                        T* rc) {
     const int czc = transfer_cz((long long)(gf.nx / 2 + 1) * (gf.ny / 2 + 1), gf.nz / 2 + 1, kRestrictCz);
     const dim3 grid((gf.nx / 2 + 1 + 31) / 32, (gf.ny / 2 + 1 + 7) / 8, (gf.nz / 2 + 1 + czc - 1) / czc);
-    if (czc == 1) k_restrict_z<T, true><<<grid, dim3(32, 8), 0, c.s>>>(maskf, maskc, rf, rc, gf.nx, gf.ny, gf.nz, czc);
+    const bool early = czc == 1 && (sizeof(T) == 4 || grid.x * grid.y * grid.z <= 2 * 152);
+    if (early) k_restrict_z<T, true><<<grid, dim3(32, 8), 0, c.s>>>(maskf, maskc, rf, rc, gf.nx, gf.ny, gf.nz, czc);
     else k_restrict_z<T, false><<<grid, dim3(32, 8), 0, c.s>>>(maskf, maskc, rf, rc, gf.nx, gf.ny, gf.nz, czc);
     TOPO_LAUNCH_CHECK(c);
 }
